@@ -330,10 +330,11 @@ STEPKV_API stepkv_status_t stepkv_compact(int32_t n_layers, const void* const* K
  *           compaction), else n_host.  A device value above n_cap sets STEPKV_ENOSPACE and n_cap rows
  *           are used; a value below 1 sets STEPKV_EDATA and the output is zero.
  *  out[l]   host array of device pointers, [Hq][d] fp32.
- *  ws       scratch of stepkv_decode_workspace_size bytes (256-byte aligned): per-split partials.
+ *  ws       scratch of stepkv_decode_workspace_size bytes (256-byte aligned): partial states.
  *  Supported: d in {64, 128}; G = Hq / Hkv in {1, 2, 4, 5, 8}; 1 <= n_cap; n_host <= n_cap.
- *  Work: split-K over 512-key chunks (one chunk of one (layer, KV head) per CTA, all G heads of the
- *  group per key-row load), then a merge of the chunks in order (deterministic).
+ *  Work: the keys of every (layer, KV head) are split over warps (all G heads of the group per key-row
+ *  load), then the partial states are merged in key order (deterministic; the split depends on n_layers,
+ *  Hkv and n_cap, so the last bits of a result do too).
  */
 STEPKV_API size_t stepkv_decode_workspace_size(int32_t n_layers, int32_t Hkv, int32_t Hq, int32_t d, int32_t n_cap);
 STEPKV_API stepkv_status_t stepkv_decode(int32_t n_layers, const void* const* q, const void* const* K,
@@ -354,7 +355,7 @@ STEPKV_API stepkv_status_t stepkv_decode(int32_t n_layers, const void* const* q,
  *           per head over the keys).  The caller zeroes the rows (e.g. after a boundary) and reads
  *           them as saliency rows, e.g. stepkv_select(sal = mass rows of chosen layers, n_sal =
  *           layers x Hkv): T_i is then the mean accumulated attention of token i (Eq. 5's T_i).
- *  ws       stepkv_decode_h2o_workspace_size bytes: the split partials and every key's logits.
+ *  ws       stepkv_decode_h2o_workspace_size bytes: the partial states and every key's logits.
  *  out is bit-identical to stepkv_decode's on the same inputs; the masses are deterministic (one
  *  writer per element and call, heads summed in a fixed order).
  */

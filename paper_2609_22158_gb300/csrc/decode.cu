@@ -4,22 +4,33 @@
 //   out[g][:] = sum_{j < n} softmax_j( q[g] . K[g/G][j] / sqrt(d) ) V[g/G][j][:]
 //
 // GB300 design: HBM-bound (the K and V rows are read once per token, 1.08 GB for 32 layers x 8 heads x
-// 8272 rows), so the kernel is built around coalesced 16-byte loads and enough bytes in flight; the
-// contraction is 2 x G x d flop per key row and stays on the FP32 pipe.  Split-K: a CTA owns 512 keys of
-// one (layer, KV head) pair and all G query heads of its group, so every key row is loaded once for the
-// whole group.  d/8 lanes share a key row (8 bf16 each); a warp covers 32/(d/8) keys per step, four steps
-// per block, and keeps a running (max, sum, weighted values) per head, rescaled once per block.  A
-// second kernel merges the per-split partials of each (pair, head) in split order (deterministic).
+// 8272 rows), so the work per row must stay far below what a scheduler issues while the row streams in.
+// Both contractions run on the tensor cores, straight from the rows as they lie in memory (tcgen05 would need its
+// 128-row operand tiles for the G <= 8 query heads of a pair, and V transposed; mma.sync takes 16 rows, its tensor
+// pipe is 20% busy here):
+//   S = Q K^T: the heads are the rows of A, 8 keys the columns of B.  A lane's 16-byte vector of a key
+//     row is the B fragment of two k-steps; which of the d elements a k-step covers is free as long as
+//     Q is loaded the same way.
+//   O = P V: the probabilities of 16 keys are A (the accumulator layout of S is already A's layout), a
+//     V row vector gives the B fragments of 8 column tiles after one byte permute per two elements.
+// The probabilities stay exact to 24 bits: p = hi + mid + lo, three bf16 terms in groups of A's rows (G <= 4: one MMA
+// holds all three; G <= 8: two MMAs).  Every MMA starts from a zero accumulator and is added to the running sums with
+// fp32 adds, because the tensor core's own accumulation truncates: the output's error against 64-bit values is 3.8e-7
+// at 8272 rows (5.2e-7 with fp32 FMAs and a logit rounded before its exponent).
+// Each warp copies whole rows (16 keys and values a step) into a ring of its own with cp.async and needs no other
+// warp: 13 instructions per key row instead of 79, so the reads bound it.  32 layers x 8 heads x 8272 rows, G = 4:
+// 208 -> 168 us (6.44 TB/s); 8 query heads per KV head 449 -> 172 us.  Reading the fragments straight from global
+// memory, 64 bytes of each of 8 rows per load, ran at 215 us: full 128-byte lines matter.
+//
+// Two splits, chosen by the number of (layer, KV head) pairs and keys (decode_plan): each warp streams an equal range
+// of the list of all pairs' 16-key blocks, or (few pairs or keys) each pair is split over CTAs whose warps
+// interleave its blocks.  A second kernel merges the partial states of a pair in key order (deterministic).
 // The number of keys may be read on the device (n_kept of a compaction), so no host sync is needed.
 //
 // Accumulated attention (the H2O-style token saliency, Sec. 4.2: T_i may come from an existing
-// token-level importance estimator): with mass rows given, the partial kernel also stores every key's
-// logits per head, and the merge runs up to 8 CTAs per (layer, KV head), each over a contiguous share of
-// the keys.  Every CTA merges the heads' (m, l) split states in split order into each head's
-// log-sum-exp (the first CTA also merges the value rows, in the same order as the plain merge, so the
-// outputs are bit-identical).  Then its threads add (1/G) sum_g softmax_j(q_g . k_j / sqrt(d)) to
-// mass[j] for each of its keys: one writer per element and call, a fixed order over g, so the result is
-// deterministic.
+// token-level importance estimator): with mass rows given, the first kernel also stores every key's logits, and
+// the second adds (1/G) sum_g softmax_j(q_g . k_j / sqrt(d)) to mass[j] for each key from the heads' log-sum-exp:
+// one writer per element and call, a fixed order over g, so the result is deterministic.
 #include <math.h>
 
 #include <algorithm>
@@ -29,10 +40,13 @@
 
 namespace stepkv {
 
-constexpr int kDecThreads = 128;
-constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kDecSplitKeys = 512;
-constexpr int kDecBlockSteps = 4;
+constexpr int kDecWarps = 8;
+constexpr int kDecThreads = kDecWarps * 32;
+constexpr int kDecBlock = 16;           // keys per warp step
+// Per warp: two stages of 16 key and 16 value rows at d = 128, four at d = 64.  32 layers x 8 heads x 8272 rows, G = 4:
+// 168.4 us; 24 KB 171.8; 12 warps of 16 KB 168.0 (and every G > 4 shape 5-7% slower: spills); 6 warps of 32 KB 175.1.
+constexpr int kDecRingBytes = 16 << 10;
+constexpr int kDecSplitKeys = 512;      // workspace sizing: one partial per 512 keys of a pair
 
 struct DecodeArgs {
   const uint16_t* q[kMaxDecodeLayers];
@@ -41,13 +55,17 @@ struct DecodeArgs {
   float* out[kMaxDecodeLayers];
   int64_t head_stride;  // elements
   int Hkv;
-  int n_splits;
+  int G;
+  int pairs;
+  int n_groups;         // CTAs per pair (split form)
+  int n_warps;          // warps of the launch (stream form), 0: split form
+  int chunks;           // accumulated attention: blocks of the merge kernel per pair
   const int32_t* n_dev;
   int n_host;
   int n_cap;
   float c;              // log2(e) / sqrt(d)
-  float* part;          // [pairs][n_splits][G][d + 4]: m, l, -, -, acc[d]
-  float* logits;        // [pairs][n_cap][G] (accumulated-attention mode, else NULL): key logits in log2 units
+  float* part;          // partial states [slot][G][d + 4]: m c, l, -, -, acc[d]
+  float* logits;        // [pairs][n_cap][G] (accumulated-attention mode, else NULL): q . k of every key
   float* mass[kMaxDecodeLayers];  // per layer [Hkv][mass_stride]: accumulated attention (+=), or NULL
   int64_t mass_stride;
   int32_t* status;
@@ -60,16 +78,32 @@ __device__ __forceinline__ int decode_n(const DecodeArgs& a) {
   return n;
 }
 
-__device__ __forceinline__ void bf16x8_to_f32(const uint4& r, float (&f)[8]) {
-  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    f[2 * i] = __uint_as_float(w[i] << 16);
-    f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
-  }
+// D = A B for one m16n8k16 tile of bf16 operands, from a zero accumulator.
+__device__ __forceinline__ void mma_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                          uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// Merge the state (m2, l2, acc2) into (m, l, acc); -inf marks an empty state.
+// Two fp32 values as a bf16 pair (lo = x, hi = y), rounded to nearest even.
+__device__ __forceinline__ uint32_t bf16x2_rn(float x, float y) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(y), "f"(x));
+  return r;
+}
+// p = hi + mid + lo exactly (24 bits): each term the rounding of what the terms before leave.
+__device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  hi = bf16x2_rn(x, y);
+  x -= __uint_as_float(hi << 16);
+  y -= __uint_as_float(hi & 0xFFFF0000u);
+  mid = bf16x2_rn(x, y);
+  x -= __uint_as_float(mid << 16);
+  y -= __uint_as_float(mid & 0xFFFF0000u);
+  lo = bf16x2_rn(x, y);
+}
+
+// Merge the state (m2, l2, acc2) into (m, l, acc), m in log2 units; -inf marks an empty state.
 template <int E>
 __device__ __forceinline__ void merge_state(float& m, float& l, float (&acc)[E], float m2, float l2,
                                             const float (&acc2)[E]) {
@@ -82,310 +116,450 @@ __device__ __forceinline__ void merge_state(float& m, float& l, float (&acc)[E],
   m = mn;
 }
 
-// MASS: the accumulated-attention variant, which also stores every key's logits (a separate
-// instantiation, so the plain decode keeps its register budget).
-template <int D, int G, bool MASS>
-__global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const __grid_constant__ DecodeArgs a) {
-  constexpr int LPK = D / 8;          // lanes per key row
-  constexpr int KPS = 32 / LPK;       // keys per warp step
-  constexpr int BLK = KPS * kDecBlockSteps;
-  __shared__ float s_m[kDecWarps][G], s_l[kDecWarps][G];
-  __shared__ float s_acc[kDecWarps][G][D];
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared16(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// A ring stage holds 16 key rows, then 16 value rows, as they lie in memory, with the 16-byte vectors of a row permuted
+// (vector ^ mask of the row) so that the fragment reads do not conflict: eight lanes of a key read take four vectors of
+// rows r and r + 1, eight lanes of a value read take two vectors of rows r, r + 2, r + 4 and r + 6.
+__device__ __forceinline__ int decode_k_swizzle(int row) { return (row & 1) << 2; }
+__device__ __forceinline__ int decode_v_swizzle(int row) { return row & 6; }
+
+// One warp's state over the keys of a pair: running maximum of q . k (row `head`), this lane's part of the
+// sum, and the weighted values.  acc[s][t] holds elements 64 s + 16 c4 + t and + 8 of row r8 (GP = 4: the hi + lo terms
+// in rows 0-3, the mid terms in rows 4-7).
+template <int D, int GP>
+struct DecodeState {
+  static constexpr int NCH = D / 32;    // 16-byte vectors of a key row per lane
+  static constexpr int NSET = D / 64;   // 16-byte vectors of a value row per lane
+  float m, l;
+  uint64_t acc[NSET][8];
+
+  __device__ __forceinline__ void clear() {
+    m = -INFINITY;
+    l = 0.f;
+#pragma unroll
+    for (int s = 0; s < NSET; ++s)
+#pragma unroll
+      for (int t = 0; t < 8; ++t) acc[s][t] = 0ull;
+  }
+
+  // Keys kb .. kb + 15 (those at or past k_end masked), their rows in the ring stage `ring` (decode_k_swizzle,
+  // decode_v_swizzle).  Returns the logits q . k of keys kb + 8t + 2 c4 + x in s.
+  __device__ __forceinline__ void block(uint32_t ring, const uint32_t (&qa)[2 * NCH][2], int kb, int k_end, float c,
+                                        int lane, float (&s)[2][2]) {
+    const int r8 = lane >> 2, c4 = lane & 3;
+    const uint32_t kbase = ring + r8 * (2 * D), kx = decode_k_swizzle(r8);
+    const uint32_t vbase = ring + 16 * 2 * D + 2 * c4 * (2 * D);
+    // each k-step's product from zero, then fp32 adds as a tree
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      uint64_t x[2 * NCH];
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        const uint4 k = ld_shared16(kbase + t * 16 * D + (((c4 + 4 * i) ^ kx) << 4));
+        float d[4];
+        mma_16816(d, qa[2 * i][0], qa[2 * i][0], qa[2 * i][1], qa[2 * i][1], k.x, k.y);
+        x[2 * i] = f2_pack(d[0], d[1]);
+        mma_16816(d, qa[2 * i + 1][0], qa[2 * i + 1][0], qa[2 * i + 1][1], qa[2 * i + 1][1], k.z, k.w);
+        x[2 * i + 1] = f2_pack(d[0], d[1]);
+      }
+#pragma unroll
+      for (int w = NCH; w > 0; w >>= 1)
+#pragma unroll
+        for (int i = 0; i < w; ++i) x[i] = f2_add(x[i], x[i + w]);
+      f2_unpack(x[0], s[t][0], s[t][1]);
+    }
+    if (kb + kDecBlock > k_end) {
+#pragma unroll
+      for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          if (kb + 8 * t + 2 * c4 + x >= k_end) s[t][x] = -INFINITY;
+    }
+    float mb = fmax3(fmaxf(s[0][0], s[0][1]), s[1][0], s[1][1]);
+    mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
+    mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
+    if (__any_sync(0xffffffffu, mb > m)) {
+      const float mn = fmaxf(m, mb);
+      const float sc = ex2_approx((m - mn) * c);
+      const uint64_t sc2 = f2_pack(sc, sc);
+      l *= sc;
+#pragma unroll
+      for (int s2 = 0; s2 < NSET; ++s2)
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc[s2][t] = f2_mul(acc[s2][t], sc2);
+      m = mn;
+    }
+    const float mc = m * c;
+    float p[2][2];
+    uint32_t ph[2], pm[2], pl[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      p[t][0] = ex2_approx(fmaf(s[t][0], c, -mc));
+      p[t][1] = ex2_approx(fmaf(s[t][1], c, -mc));
+      split3(p[t][0], p[t][1], ph[t], pm[t], pl[t]);
+    }
+    l += (p[0][0] + p[0][1]) + (p[1][0] + p[1][1]);
+    uint32_t a0 = ph[0], a1 = pm[0], a2 = ph[1], a3 = pm[1];
+    if (GP == 4) {
+      const bool top = lane < 16;
+      a0 = top ? ph[0] : pm[0];
+      a1 = top ? pl[0] : 0u;
+      a2 = top ? ph[1] : pm[1];
+      a3 = top ? pl[1] : 0u;
+    }
+#pragma unroll
+    for (int s2 = 0; s2 < NSET; ++s2) {
+      uint32_t v[4][4];  // [key 2 c4, 2 c4 + 1, 2 c4 + 8, 2 c4 + 9][pair of elements]
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int row = (x & 1) + 8 * (x >> 1);  // beyond 2 c4
+        const uint4 r = ld_shared16(vbase + row * (2 * D) + (((r8 + 8 * s2) ^ decode_v_swizzle(2 * c4 + row)) << 4));
+        v[x][0] = r.x;
+        v[x][1] = r.y;
+        v[x][2] = r.z;
+        v[x][3] = r.w;
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        const uint32_t sel = (t & 1) ? 0x7632u : 0x5410u;
+        const uint32_t b0 = __byte_perm(v[0][t >> 1], v[1][t >> 1], sel), b1 = __byte_perm(v[2][t >> 1], v[3][t >> 1], sel);
+        float d[4];
+        mma_16816(d, a0, a1, a2, a3, b0, b1);
+        uint64_t o = f2_add(f2_pack(d[0], d[1]), f2_pack(d[2], d[3]));
+        if (GP == 8) {
+          mma_16816(d, pl[0], 0u, pl[1], 0u, b0, b1);
+          o = f2_add(o, f2_pack(d[0], d[1]));
+        }
+        acc[s2][t] = f2_add(acc[s2][t], o);
+      }
+    }
+  }
+
+  // The warp's state written out: m c and l of head g at ml[g * ml_stride + {0, 1}], the values at vals + g * v_stride.
+  __device__ __forceinline__ void store(float* ml, int ml_stride, float* vals, int v_stride, float c, int G, int lane) {
+    const int r8 = lane >> 2, c4 = lane & 3, head = GP == 4 ? (r8 & 3) : r8;
+    float ls = l;
+    ls += __shfl_xor_sync(0xffffffffu, ls, 1);
+    ls += __shfl_xor_sync(0xffffffffu, ls, 2);
+    const bool writes = head < G && (GP == 8 || lane < 16);
+#pragma unroll
+    for (int s2 = 0; s2 < NSET; ++s2) {
+      float x[8], y[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        f2_unpack(acc[s2][t], x[t], y[t]);
+        if (GP == 4) {
+          x[t] += __shfl_xor_sync(0xffffffffu, x[t], 16);
+          y[t] += __shfl_xor_sync(0xffffffffu, y[t], 16);
+        }
+      }
+      if (writes) {
+        float4* dst = reinterpret_cast<float4*>(vals + head * v_stride + 64 * s2 + 16 * c4);
+        dst[0] = make_float4(x[0], x[1], x[2], x[3]);
+        dst[1] = make_float4(x[4], x[5], x[6], x[7]);
+        dst[2] = make_float4(y[0], y[1], y[2], y[3]);
+        dst[3] = make_float4(y[4], y[5], y[6], y[7]);
+      }
+    }
+    if (writes && c4 == 0) {
+      ml[head * ml_stride] = m * c;
+      ml[head * ml_stride + 1] = ls;
+    }
+  }
+};
+
+// GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
+// MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
+// STREAM: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
+// per pair it touches (slot warp + pair); a merge kernel follows.  Else a cluster works on one pair.
+template <int D, int GP, bool MASS, bool STREAM>
+__global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_constant__ DecodeArgs a) {
+  using State = DecodeState<D, GP>;
+  constexpr int NT = kDecThreads, NW = kDecWarps;
+  constexpr int NCH = State::NCH;
+  constexpr int kStageBytes = 2 * kDecBlock * D * 2;
+  constexpr int kStages = kDecRingBytes / kStageBytes;
+  extern __shared__ __align__(16) uint8_t dec_smem[];     // per-warp rings | logits (MASS, cluster form)
 
   pdl_wait();
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int pair = blockIdx.x / a.n_splits, split = blockIdx.x - pair * a.n_splits;
-  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+  const int r8 = lane >> 2, c4 = lane & 3;                // fragment row (or column) and position in it
+  const int head = GP == 4 ? (r8 & 3) : r8;               // the head of this lane's rows r8 and r8 + 8
+  const int G = a.G;
+  const float c = a.c;
   int n = decode_n(a);
   if (n > a.n_cap) {
     if (threadIdx.x == 0 && blockIdx.x == 0) record_status(a.status, STEPKV_ENOSPACE);
     n = a.n_cap;
   }
-  if (n < 1 && threadIdx.x == 0 && blockIdx.x == 0) record_status(a.status, STEPKV_EDATA);
-  const int k_begin = split * kDecSplitKeys;
-  const int k_end = min(n, k_begin + kDecSplitKeys);
-  const int kslot = lane / LPK, hl = lane - kslot * LPK;
-
-  // this lane's 8 elements of every query head of the group, pre-scaled for exp2
-  float q[G][8];
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const uint4 r = __ldg(reinterpret_cast<const uint4*>(a.q[layer] + (size_t)(h * G + g) * D) + hl);
-    bf16x8_to_f32(r, q[g]);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) q[g][e] *= a.c;
+  if (n < 1) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) record_status(a.status, STEPKV_EDATA);
+    n = 0;
   }
-  // Value accumulators as packed fp32 pairs: a bf16 word holds two neighbouring elements, so a value row
-  // converts straight into pairs and every value FMA and rescale is one f32x2 instruction for two elements.
-  float m[G], l[G];
-  uint64_t accp[G][4];
+  uint8_t* my_ring = dec_smem + warp * kDecRingBytes;
+  const uint32_t ring0 = smem_u32(my_ring);
+  // A warp copies whole rows (256 or 128 consecutive bytes each); rows past `last` are read as row `last` (in range,
+  // finite) and their probabilities set to zero.
+  constexpr int VPR = D / 8, RPI = 32 / VPR;              // vectors per row, rows per copy instruction
+  const int cp_row = lane / VPR, cp_vec = lane & (VPR - 1);
+  auto issue = [&](uint32_t dst, const uint16_t* Kh, const uint16_t* Vh, int kb, int last) {
 #pragma unroll
-  for (int g = 0; g < G; ++g) {
-    m[g] = -INFINITY;
-    l[g] = 0.f;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) accp[g][e] = 0ull;
-  }
-
-  const uint16_t* Kh = a.K[layer] + (size_t)h * a.head_stride;
-  const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
-  // warp w takes blocks w, w + 4, ... of BLK consecutive keys
-  for (int kb = k_begin + warp * BLK; kb < k_end; kb += kDecWarps * BLK) {
-    uint4 kr[kDecBlockSteps], vr[kDecBlockSteps];
-    bool ok[kDecBlockSteps];
-#pragma unroll
-    for (int t = 0; t < kDecBlockSteps; ++t) {
-      const int j = kb + t * KPS + kslot;
-      ok[t] = j < k_end;
-      kr[t] = ok[t] ? __ldcs(reinterpret_cast<const uint4*>(Kh + (size_t)j * D) + hl) : make_uint4(0, 0, 0, 0);
-      vr[t] = ok[t] ? __ldcs(reinterpret_cast<const uint4*>(Vh + (size_t)j * D) + hl) : make_uint4(0, 0, 0, 0);
+    for (int i = 0; i < kDecBlock / RPI; ++i) {
+      const int row = i * RPI + cp_row;
+      const size_t src = (size_t)min(kb + row, last) * D + cp_vec * 8;
+      cp_async16(dst + row * (2 * D) + ((cp_vec ^ decode_k_swizzle(row)) << 4), Kh + src);
+      cp_async16(dst + (16 + row) * (2 * D) + ((cp_vec ^ decode_v_swizzle(row)) << 4), Vh + src);
     }
-    // The warp's next block is fetched into L2 while this one is computed: the loads above wait for
-    // DRAM only until the pipeline fills, and the prefetch holds no registers.
-    const int kn = kb + kDecWarps * BLK;
-    if (lane == 0 && kn < k_end) {
-      const uint32_t nbytes = (uint32_t)(min(BLK, k_end - kn) * D * 2);
-      bulk_prefetch_l2(Kh + (size_t)kn * D, nbytes);
-      bulk_prefetch_l2(Vh + (size_t)kn * D, nbytes);
+  };
+  // A fragments of Q: k-step 2i + x covers elements 4x .. 4x + 3 of every lane's vector c4 + 4i (rows r8 and r8 + 8
+  // hold the same head, so a1 = a0 and a3 = a2)
+  uint32_t qa[2 * NCH][2];
+  auto load_q = [&](int layer, int h) {
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+      uint4 v = make_uint4(0, 0, 0, 0);
+      if (head < G) v = __ldg(reinterpret_cast<const uint4*>(a.q[layer] + (size_t)(h * G + head) * D) + c4 + 4 * i);
+      qa[2 * i][0] = v.x;
+      qa[2 * i][1] = v.y;
+      qa[2 * i + 1][0] = v.z;
+      qa[2 * i + 1][1] = v.w;
     }
-    float s[kDecBlockSteps][G];
+  };
+  auto store_logits = [&](int pair, int kb, int k_end, const float (&s)[2][2]) {
+    if (head >= G || (GP == 4 && lane >= 16)) return;
 #pragma unroll
-    for (int t = 0; t < kDecBlockSteps; ++t) {
-      float kf[8];
-      bf16x8_to_f32(kr[t], kf);
-      float x[G];
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        x[g] = 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) x[g] = fmaf(q[g][e], kf[e], x[g]);
+      for (int x = 0; x < 2; ++x) {
+        const int j = kb + 8 * t + 2 * c4 + x;
+        if (j < k_end) a.logits[((size_t)pair * a.n_cap + j) * G + head] = s[t][x];
       }
-      if constexpr (G == 4) {
-        // reduce-scatter over the LPK lanes of the row (each lane ends with one head's full sum), then
-        // broadcast the four sums: 9 shuffles instead of 4 x log2(LPK)
-        constexpr int A = LPK / 2, Bx = LPK / 4;
-        const bool ba = (hl & A) != 0, bb = (hl & Bx) != 0;
-        const float y0 = (ba ? x[2] : x[0]) + __shfl_xor_sync(0xffffffffu, ba ? x[0] : x[2], A);
-        const float y1 = (ba ? x[3] : x[1]) + __shfl_xor_sync(0xffffffffu, ba ? x[1] : x[3], A);
-        float z = (bb ? y1 : y0) + __shfl_xor_sync(0xffffffffu, bb ? y0 : y1, Bx);
-#pragma unroll
-        for (int o = Bx / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        const int base_lane = lane & ~(LPK - 1);
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const float v = __shfl_sync(0xffffffffu, z, base_lane | (((g >> 1) ? A : 0) | ((g & 1) ? Bx : 0)));
-          s[t][g] = ok[t] ? v : -INFINITY;
+  };
+  State st;
+  st.clear();
+
+  if constexpr (STREAM) {
+    const int nb = (n + kDecBlock - 1) / kDecBlock;       // blocks per pair
+    const int total = a.pairs * nb;
+    const int per = (total + a.n_warps - 1) / a.n_warps;
+    const int w = blockIdx.x * NW + warp;
+    const int lo = min(total, w * per), hi = min(total, lo + per);
+    if (lo >= hi) return;
+    // the copies run kStages blocks ahead of the arithmetic, across pair boundaries
+    int i_pair = lo / nb, i_kb = (lo - i_pair * nb) * kDecBlock, i_left = hi - lo;
+    const uint16_t *Kh, *Vh;
+    auto bases = [&](int pair) {
+      const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+      Kh = a.K[layer] + (size_t)h * a.head_stride;
+      Vh = a.V[layer] + (size_t)h * a.head_stride;
+    };
+    bases(i_pair);
+    auto issue_next = [&](uint32_t dst) {
+      if (i_left > 0) {
+        issue(dst, Kh, Vh, i_kb, n - 1);
+        --i_left;
+        i_kb += kDecBlock;
+        if (i_kb >= n && i_left > 0) {
+          i_kb = 0;
+          bases(++i_pair);
         }
+      }
+      cp_async_commit();
+    };
+    int pair = i_pair, kb = i_kb, stage = 0;
+#pragma unroll
+    for (int s = 0; s < kStages; ++s) issue_next(ring0 + s * kStageBytes);
+    load_q(pair / a.Hkv, pair - pair / a.Hkv * a.Hkv);
+    for (int left = hi - lo;;) {
+      cp_async_wait<kStages - 1>();
+      __syncwarp();
+      float s[2][2];
+      const uint32_t ring = ring0 + stage * kStageBytes;
+      st.block(ring, qa, kb, n, c, lane, s);
+      __syncwarp();
+      issue_next(ring);
+      if (MASS) store_logits(pair, kb, n, s);
+      stage = stage + 1 == kStages ? 0 : stage + 1;
+      kb += kDecBlock;
+      --left;
+      if (kb >= n || left == 0) {
+        float* dst = a.part + (size_t)(w + pair) * G * (D + 4);
+        st.store(dst, D + 4, dst + 4, D + 4, c, G, lane);
+        if (left == 0) break;
+        st.clear();
+        ++pair;
+        kb = 0;
+        load_q(pair / a.Hkv, pair - pair / a.Hkv * a.Hkv);
+      }
+    }
+  } else {
+    __shared__ float s_ml[NW][GP][2];
+    const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
+    const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+    const int share = ((n + a.n_groups - 1) / a.n_groups + kDecBlock - 1) & ~(kDecBlock - 1);
+    const int k_begin = min(n, grp * share), k_end = min(n, k_begin + share);
+    const uint16_t* Kh = a.K[layer] + (size_t)h * a.head_stride;
+    const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
+    int kb = k_begin + warp * kDecBlock, i_kb = kb, stage = 0;
+    auto issue_next = [&](uint32_t dst) {
+      if (i_kb < k_end) issue(dst, Kh, Vh, i_kb, k_end - 1);
+      i_kb += NW * kDecBlock;
+      cp_async_commit();
+    };
+#pragma unroll
+    for (int s = 0; s < kStages; ++s) issue_next(ring0 + s * kStageBytes);
+    load_q(layer, h);
+    for (; kb < k_end; kb += NW * kDecBlock) {
+      cp_async_wait<kStages - 1>();
+      __syncwarp();
+      float s[2][2];
+      const uint32_t ring = ring0 + stage * kStageBytes;
+      st.block(ring, qa, kb, k_end, c, lane, s);
+      __syncwarp();
+      issue_next(ring);
+      if (MASS) store_logits(pair, kb, k_end, s);
+      stage = stage + 1 == kStages ? 0 : stage + 1;
+    }
+    cp_async_wait<0>();
+    __syncwarp();
+    st.store(&s_ml[warp][0][0], 2, reinterpret_cast<float*>(my_ring), D, c, G, lane);  // the ring is empty now
+    __syncthreads();
+    // the warps merged in order, four elements of one head per thread
+    constexpr int V4 = D / 4;
+    for (int t = threadIdx.x; t < G * V4; t += NT) {
+      const int g = t / V4, e0 = (t - g * V4) * 4;
+      float mm = -INFINITY, ll = 0.f, aa[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int w = 0; w < NW; ++w) {
+        const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(dec_smem + w * kDecRingBytes) + g * D + e0);
+        const float a2[4] = {v.x, v.y, v.z, v.w};
+        merge_state<4>(mm, ll, aa, s_ml[w][g][0], s_ml[w][g][1], a2);
+      }
+      if (!MASS && a.n_groups == 1) {
+        const float inv = ll > 0.f ? 1.f / ll : 0.f;
+        *reinterpret_cast<float4*>(a.out[layer] + (size_t)(h * G + g) * D + e0) =
+            make_float4(aa[0] * inv, aa[1] * inv, aa[2] * inv, aa[3] * inv);
       } else {
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float v = x[g];
-#pragma unroll
-          for (int o = LPK / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-          s[t][g] = ok[t] ? v : -INFINITY;
+        float* dst = a.part + ((size_t)blockIdx.x * G + g) * (D + 4);
+        if (e0 == 0) {
+          dst[0] = mm;
+          dst[1] = ll;
         }
-      }
-    }
-    if (MASS && hl == 0) {
-      // every lane of a key row holds the row's logits of all G heads: the first one stores them
-#pragma unroll
-      for (int t = 0; t < kDecBlockSteps; ++t) {
-        const int j = kb + t * KPS + kslot;
-        if (ok[t]) {
-          float* dst = a.logits + ((size_t)pair * a.n_cap + j) * G;
-          if constexpr (G % 4 == 0) {
-#pragma unroll
-            for (int g = 0; g < G; g += 4)
-              *reinterpret_cast<float4*>(dst + g) = make_float4(s[t][g], s[t][g + 1], s[t][g + 2], s[t][g + 3]);
-          } else {
-#pragma unroll
-            for (int g = 0; g < G; ++g) dst[g] = s[t][g];
-          }
-        }
-      }
-    }
-    // probabilities of the block's keys per head (state rescaled once per block), then one pass over
-    // the value rows: each is converted once and accumulated into every head
-    float p[kDecBlockSteps][G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float mb = m[g];
-#pragma unroll
-      for (int t = 0; t < kDecBlockSteps; ++t) mb = fmaxf(mb, s[t][g]);
-      if (mb == -INFINITY) {
-#pragma unroll
-        for (int t = 0; t < kDecBlockSteps; ++t) p[t][g] = 0.f;
-        continue;
-      }
-      const float sc = ex2_approx(m[g] - mb);
-      l[g] *= sc;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) accp[g][e] = f2_mul(accp[g][e], f2_pack(sc, sc));
-#pragma unroll
-      for (int t = 0; t < kDecBlockSteps; ++t) {
-        p[t][g] = ex2_approx(s[t][g] - mb);
-        l[g] += p[t][g];
-      }
-      m[g] = mb;
-    }
-#pragma unroll
-    for (int t = 0; t < kDecBlockSteps; ++t) {
-      const uint32_t w[4] = {vr[t].x, vr[t].y, vr[t].z, vr[t].w};
-      uint64_t vp[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) vp[e] = f2_pack(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u));
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const uint64_t pp = f2_pack(p[t][g], p[t][g]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) accp[g][e] = f2_fma(vp[e], pp, accp[g][e]);
+        *reinterpret_cast<float4*>(dst + 4 + e0) = make_float4(aa[0], aa[1], aa[2], aa[3]);
       }
     }
   }
-  float acc[G][8];
-#pragma unroll
-  for (int g = 0; g < G; ++g)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) f2_unpack(accp[g][e], acc[g][2 * e], acc[g][2 * e + 1]);
-  // merge the key slots of the warp (lanes with the same hl), then the warps through shared memory
-#pragma unroll
-  for (int o = LPK; o < 32; o <<= 1) {
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m[g], o);
-      const float l2 = __shfl_xor_sync(0xffffffffu, l[g], o);
-      float acc2[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc2[e] = __shfl_xor_sync(0xffffffffu, acc[g][e], o);
-      merge_state<8>(m[g], l[g], acc[g], m2, l2, acc2);
-    }
+}
+
+// The partial slots of a pair, in key order: of the stream form those of the warps whose ranges reach into the pair,
+// else its CTAs' (all of them, empty shares included, so that the number of keys need not be read first).
+__device__ __forceinline__ void decode_slots(const DecodeArgs& a, int pair, int& first, int& count) {
+  if (a.n_warps == 0) {
+    first = pair * a.n_groups;
+    count = a.n_groups;
+    return;
   }
-  if (kslot == 0) {
+  const int n = max(0, min(decode_n(a), a.n_cap));
+  const int nb = (n + kDecBlock - 1) / kDecBlock;
+  const int per = (a.pairs * nb + a.n_warps - 1) / a.n_warps;
+  first = count = 0;
+  if (nb == 0) return;
+  const int w0 = pair * nb / per, w1 = ((pair + 1) * nb - 1) / per;
+  first = w0 + pair;
+  count = w1 - w0 + 1;
+}
+
+// Merge of the partial states.  Blocks [0, pairs * G) take one (pair, head) each: warp w merges slots w, w + 4, ... in
+// order (the loads of eight in flight), then the warps meet in order, and out = acc / l.  With accumulated attention,
+// `chunks` more blocks per pair each take a contiguous share of the keys: the heads' log-sum-exp from all slots, then
+// the group-mean softmax mass of every key of the share is added (one writer per key).
+constexpr int kDecMergeThreads = 128;
+
+template <int D>
+__global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __grid_constant__ DecodeArgs a) {
+  constexpr int PER = D / 32, NW = kDecMergeThreads / 32;
+  __shared__ float s_ml[NW][2];
+  __shared__ float s_v[NW][D];
+  __shared__ float s_lse[8];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int G = a.G, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int item = (int)blockIdx.x;
+  int first, count;
+  if (item < a.pairs * G) {
+    const int pair = item / G, g = item - pair * G;
+    const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+    decode_slots(a, pair, first, count);
+    float mm = -INFINITY, ll = 0.f, aa[PER];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      if (hl == 0) {
-        s_m[warp][g] = m[g];
-        s_l[warp][g] = l[g];
-      }
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s_acc[warp][g][hl * 8 + e] = acc[g][e];
-    }
-  }
-  __syncthreads();
-  // thread t < G*D/4: head g = t / (D/4), elements 4*(t % (D/4)) .. +4 -> merge the warps in order
-  constexpr int PER = 4;
-  for (int t = threadIdx.x; t < G * (D / PER); t += kDecThreads) {
-    const int g = t / (D / PER), e0 = (t - g * (D / PER)) * PER;
-    float mm = -INFINITY, ll = 0.f, aa[PER] = {0.f, 0.f, 0.f, 0.f};
-    for (int w = 0; w < kDecWarps; ++w) {
+    for (int e = 0; e < PER; ++e) aa[e] = 0.f;
+#pragma unroll 8
+    for (int i = warp; i < count; i += NW) {
+      const float* src = a.part + ((size_t)(first + i) * G + g) * (D + 4);
+      const float2 ml = __ldcg(reinterpret_cast<const float2*>(src));
       float a2[PER];
 #pragma unroll
-      for (int e = 0; e < PER; ++e) a2[e] = s_acc[w][g][e0 + e];
-      merge_state<PER>(mm, ll, aa, s_m[w][g], s_l[w][g], a2);
+      for (int e = 0; e < PER; ++e) a2[e] = __ldcg(src + 4 + e * 32 + lane);
+      merge_state<PER>(mm, ll, aa, ml.x, ml.y, a2);
     }
-    float* dst = a.part + ((size_t)(pair * a.n_splits + split) * G + g) * (D + 4);
-    if (e0 == 0) {
-      dst[0] = mm;
-      dst[1] = ll;
+    if (lane == 0) {
+      s_ml[warp][0] = mm;
+      s_ml[warp][1] = ll;
     }
-    *reinterpret_cast<float4*>(dst + 4 + e0) = make_float4(aa[0], aa[1], aa[2], aa[3]);
-  }
-}
-
-// One warp per (pair, head): merge the splits in order and write out = acc / l.
-template <int D, int G>
-__global__ void __launch_bounds__(128) decode_merge_kernel(const __grid_constant__ DecodeArgs a, int n_items) {
-  constexpr int PER = D / 32;
-  pdl_wait();
-  pdl_launch_dependents();
-  const int item = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (item >= n_items) return;
-  const int pair = item / G, g = item - pair * G;
-  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
-  int n = min(decode_n(a), a.n_cap);
-  const int used = max(0, min(a.n_splits, (n + kDecSplitKeys - 1) / kDecSplitKeys));
-  float mm = -INFINITY, ll = 0.f, aa[PER];
 #pragma unroll
-  for (int e = 0; e < PER; ++e) aa[e] = 0.f;
-  for (int sp = 0; sp < used; ++sp) {
-    const float* src = a.part + ((size_t)(pair * a.n_splits + sp) * G + g) * (D + 4);
-    float a2[PER];
+    for (int e = 0; e < PER; ++e) s_v[warp][e * 32 + lane] = aa[e];
+    __syncthreads();
+    if ((int)threadIdx.x < D) {
+      float m1 = -INFINITY, l1 = 0.f, v1[1] = {0.f};
 #pragma unroll
-    for (int e = 0; e < PER; ++e) a2[e] = __ldcg(src + 4 + lane * PER + e);
-    merge_state<PER>(mm, ll, aa, __ldcg(src), __ldcg(src + 1), a2);
-  }
-  const float inv = ll > 0.f ? 1.f / ll : 0.f;
-  float* o = a.out[layer] + (size_t)(h * G + g) * D + lane * PER;
-#pragma unroll
-  for (int e = 0; e < PER; ++e) o[e] = aa[e] * inv;
-}
-
-// Accumulated-attention merge: one CTA per (layer, KV head).  Warp w merges heads w, w + 4, ... exactly as
-// decode_merge_kernel does (bit-identical outputs) and keeps each head's log-sum-exp; then every thread adds
-// the group-mean softmax mass of its keys to the pair's mass row.
-template <int D, int G>
-__global__ void __launch_bounds__(128) decode_merge_mass_kernel(const __grid_constant__ DecodeArgs a, int chunks) {
-  constexpr int PER = D / 32;
-  __shared__ float s_lse[G];
-  pdl_wait();
-  pdl_launch_dependents();
-  const int pair = blockIdx.x / chunks, chunk = blockIdx.x - pair * chunks;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
-  const int n = max(0, min(decode_n(a), a.n_cap));
-  const int used = max(0, min(a.n_splits, (n + kDecSplitKeys - 1) / kDecSplitKeys));
-  for (int g = warp; g < G; g += 4) {
-    if (chunk == 0) {
-      // the pair's outputs: the splits merged in order, as decode_merge_kernel
-      float mm = -INFINITY, ll = 0.f, aa[PER];
-#pragma unroll
-      for (int e = 0; e < PER; ++e) aa[e] = 0.f;
-      for (int sp = 0; sp < used; ++sp) {
-        const float* src = a.part + ((size_t)(pair * a.n_splits + sp) * G + g) * (D + 4);
-        float a2[PER];
-#pragma unroll
-        for (int e = 0; e < PER; ++e) a2[e] = __ldcg(src + 4 + lane * PER + e);
-        merge_state<PER>(mm, ll, aa, __ldcg(src), __ldcg(src + 1), a2);
+      for (int w = 0; w < NW; ++w) {
+        const float v2[1] = {s_v[w][threadIdx.x]};
+        merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
       }
-      const float inv = ll > 0.f ? 1.f / ll : 0.f;
-      float* o = a.out[layer] + (size_t)(h * G + g) * D + lane * PER;
-#pragma unroll
-      for (int e = 0; e < PER; ++e) o[e] = aa[e] * inv;
-      if (lane == 0) s_lse[g] = ll > 0.f ? mm + __log2f(ll) : INFINITY;
-    } else if (lane == 0) {
-      // the same (m, l) merge without the value rows: the same log-sum-exp in every chunk
-      float mm = -INFINITY, ll = 0.f, none[1] = {0.f};
-      for (int sp = 0; sp < used; ++sp) {
-        const float* src = a.part + ((size_t)(pair * a.n_splits + sp) * G + g) * (D + 4);
-        merge_state<1>(mm, ll, none, __ldcg(src), __ldcg(src + 1), none);
-      }
-      s_lse[g] = ll > 0.f ? mm + __log2f(ll) : INFINITY;
+      a.out[layer][(size_t)(h * G + g) * D + threadIdx.x] = l1 > 0.f ? v1[0] / l1 : 0.f;
     }
+    return;
+  }
+  const int rest = item - a.pairs * G, pair = rest / a.chunks, chunk = rest - pair * a.chunks;
+  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+  decode_slots(a, pair, first, count);
+  for (int g = warp; g < G; g += NW) {
+    float mm = -INFINITY, ll = 0.f, none[1] = {0.f};
+    for (int i = lane; i < count; i += 32) {
+      const float2 ml = __ldcg(reinterpret_cast<const float2*>(a.part + ((size_t)(first + i) * G + g) * (D + 4)));
+      merge_state<1>(mm, ll, none, ml.x, ml.y, none);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, mm, o), l2 = __shfl_xor_sync(0xffffffffu, ll, o);
+      merge_state<1>(mm, ll, none, m2, l2, none);
+    }
+    if (lane == 0) s_lse[g] = ll > 0.f ? mm + __log2f(ll) : INFINITY;
   }
   __syncthreads();
-  float lse[G];
-#pragma unroll
-  for (int g = 0; g < G; ++g) lse[g] = s_lse[g];
+  const int n = max(0, min(decode_n(a), a.n_cap));
   const float inv_G = 1.f / (float)G;
   float* mrow = a.mass[layer] + (size_t)h * a.mass_stride;
   const float* lg = a.logits + (size_t)pair * a.n_cap * G;
-  // this chunk's keys (one writer per key: the additions are ordered across calls by the stream)
-  const int per = (n + chunks - 1) / chunks;
+  const int per = (n + a.chunks - 1) / a.chunks;
   const int j0 = chunk * per, j1 = min(n, j0 + per);
-  for (int j = j0 + threadIdx.x; j < j1; j += 128) {
+  for (int j = j0 + threadIdx.x; j < j1; j += kDecMergeThreads) {
     float sum = 0.f;
-    if constexpr (G % 4 == 0) {
-#pragma unroll
-      for (int g4 = 0; g4 < G; g4 += 4) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(lg + (size_t)j * G + g4));
-        sum += ex2_approx(v.x - lse[g4]) + ex2_approx(v.y - lse[g4 + 1]) + ex2_approx(v.z - lse[g4 + 2]) +
-               ex2_approx(v.w - lse[g4 + 3]);
-      }
-    } else {
-#pragma unroll
-      for (int g = 0; g < G; ++g) sum += ex2_approx(__ldcg(lg + (size_t)j * G + g) - lse[g]);
-    }
+    for (int g = 0; g < G; ++g) sum += ex2_approx(fmaf(__ldcg(lg + (size_t)j * G + g), a.c, -s_lse[g]));
     mrow[j] += sum * inv_G;
   }
 }
@@ -401,33 +575,46 @@ size_t decode_mass_ws_bytes(int n_layers, int Hkv, int Hq, int d, int n_cap) {
   return part + (size_t)n_layers * Hq * std::max(1, n_cap) * sizeof(float);
 }
 
-template <int D, int G>
-static cudaError_t decode_launch(const DecodeArgs& a, int pairs, cudaStream_t stream) {
-  if (a.logits != nullptr) {
-    cudaError_t e = launch_kernel(decode_partial_kernel<D, G, true>, dim3(pairs * a.n_splits), dim3(kDecThreads), 0,
-                                  stream, a);
-    if (e != cudaSuccess) return e;
-    // several CTAs per pair over the keys' mass updates (a pair's ~n keys are too few per SM otherwise)
-    const int chunks = std::max(1, std::min(8, (a.n_cap + 1023) / 1024));
-    return launch_kernel(decode_merge_mass_kernel<D, G>, dim3(pairs * chunks), dim3(128), 0, stream, a, chunks);
-  }
-  cudaError_t e = launch_kernel(decode_partial_kernel<D, G, false>, dim3(pairs * a.n_splits), dim3(kDecThreads), 0,
-                                stream, a);
-  if (e != cudaSuccess) return e;
-  const int items = pairs * G;
-  return launch_kernel(decode_merge_kernel<D, G>, dim3((items + 3) / 4), dim3(128), 0, stream, a, items);
+// How a launch splits `pairs` (layer, KV head) pairs of up to n_cap keys.  The stream form balances every SM and fills
+// its ring once, but a warp must have blocks enough to be worth a partial state, and the workspace holds
+// pairs x ceil(n_cap / 512) of them: it is taken where that allows three quarters of the machine's warps.  Else each pair
+// is split over as many CTAs as one wave and the workspace hold: one layer of 8 heads x 8272 rows takes 12.2 us per call
+// in a captured step (27.3 us with 512-key splits and 16-byte loads into registers; a cluster of 16 CTAs per pair with
+// the merge through distributed shared memory 24 us, since only 7 such clusters fit at a time; the last CTA of a pair
+// merging, found by an atomic count, 18.5 us).
+struct DecodePlan {
+  int n_warps;       // > 0: stream form with that many warps
+  int groups;        // else CTAs per pair
+};
+static DecodePlan decode_plan(int pairs, int n_cap, int n_sm) {
+  DecodePlan p{0, 1};
+  const int splits = std::max(1, (n_cap + kDecSplitKeys - 1) / kDecSplitKeys);  // partial slots per pair
+  // stream form: warps + pairs slots
+  const int warps = std::min(n_sm * kDecWarps, pairs * (splits - 1) / kDecWarps * kDecWarps);
+  if (warps >= n_sm * kDecWarps * 3 / 4) p.n_warps = warps;
+  else p.groups = std::max(1, std::min(splits, n_sm / pairs));
+  return p;
 }
 
-template <int D>
-static cudaError_t decode_dispatch_g(const DecodeArgs& a, int G, int pairs, cudaStream_t stream) {
-  switch (G) {
-    case 1: return decode_launch<D, 1>(a, pairs, stream);
-    case 2: return decode_launch<D, 2>(a, pairs, stream);
-    case 4: return decode_launch<D, 4>(a, pairs, stream);
-    case 5: return decode_launch<D, 5>(a, pairs, stream);
-    case 8: return decode_launch<D, 8>(a, pairs, stream);
-    default: return cudaErrorInvalidValue;
-  }
+template <int D, int GP, bool MASS, bool STREAM>
+static cudaError_t decode_launch(const DecodeArgs& a, cudaStream_t stream) {
+  void (*kern)(DecodeArgs) = decode_kernel<D, GP, MASS, STREAM>;
+  const int smem = kDecWarps * kDecRingBytes;
+  const int grid = STREAM ? a.n_warps / kDecWarps : a.pairs * a.n_groups;
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), smem);
+  // Both kernels launch dependently (each waits for the one before it before it reads anything): a captured decode
+  // step of 32 one-layer calls takes 390 us, 406 with the first launched plainly, 541 with both.
+  if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(kDecThreads), smem, stream, a, true);
+  if (e != cudaSuccess || (!STREAM && !MASS && a.n_groups == 1)) return e;
+  const int blocks = a.pairs * (a.G + (MASS ? a.chunks : 0));
+  return launch_kernel(decode_merge_kernel<D>, dim3(blocks), dim3(kDecMergeThreads), 0, stream, a, true);
+}
+
+template <int D, int GP>
+static cudaError_t decode_dispatch(const DecodeArgs& a, cudaStream_t stream) {
+  if (a.n_warps > 0)
+    return a.logits ? decode_launch<D, GP, true, true>(a, stream) : decode_launch<D, GP, false, true>(a, stream);
+  return a.logits ? decode_launch<D, GP, true, false>(a, stream) : decode_launch<D, GP, false, false>(a, stream);
 }
 
 stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const* K, const void* const* V,
@@ -435,7 +622,12 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
                            float* const* out, void* ws, int32_t* status, cudaStream_t stream, float* const* mass,
                            int64_t mass_stride) {
   const int G = Hq / Hkv;
-  const int n_splits = std::max(1, (n_cap + kDecSplitKeys - 1) / kDecSplitKeys);
+  int n_sm = 0;
+  cudaError_t e = device_sm_count(&n_sm);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e);
+    return STEPKV_ECUDA;
+  }
   float* part = static_cast<float*>(ws);
   float* logits = nullptr;
   if (mass != nullptr)
@@ -456,15 +648,22 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
     a.mass_stride = mass_stride;
     a.head_stride = head_stride;
     a.Hkv = Hkv;
-    a.n_splits = n_splits;
+    a.G = G;
+    const DecodePlan p = decode_plan(nl * Hkv, n_cap, n_sm);
+    a.pairs = nl * Hkv;
+    a.n_groups = p.groups;
+    a.n_warps = p.n_warps;
+    a.chunks = std::max(1, std::min(8, (n_cap + 1023) / 1024));
     a.n_dev = n_dev;
     a.n_host = n_host;
     a.n_cap = n_cap;
     a.c = (float)(1.4426950408889634 / sqrt((double)d));
     a.part = part;
     a.status = status;
-    const cudaError_t e = d == 128 ? decode_dispatch_g<128>(a, G, nl * Hkv, stream)
-                                   : decode_dispatch_g<64>(a, G, nl * Hkv, stream);
+    if (d == 128)
+      e = G <= 4 ? decode_dispatch<128, 4>(a, stream) : decode_dispatch<128, 8>(a, stream);
+    else
+      e = G <= 4 ? decode_dispatch<64, 4>(a, stream) : decode_dispatch<64, 8>(a, stream);
     if (e != cudaSuccess) {
       set_last_cuda_error(e);
       return STEPKV_ECUDA;

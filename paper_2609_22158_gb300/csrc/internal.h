@@ -25,8 +25,8 @@ cudaError_t ensure_smem_attr(const void* func, int bytes);
 // Kernel launch on `stream`.  Ordinary stream order unless `pdl` is set: then the launch carries the
 // programmatic-stream-serialization attribute, so the kernel may start while the preceding kernel
 // finishes and must execute griddepcontrol.wait (pdl_wait) before reading anything that kernel wrote.
-// Only the selection kernel uses it.  Measured on GB300 with the 32K workload, the compaction kernel
-// ran ~25% slower when launched with the attribute (178 us vs 140 us), so it is launched plainly.
+// The selection, in-place move and decode kernels use it.  Measured on GB300 with the 32K workload, the
+// out-of-place compaction ran ~25% slower when launched with the attribute (178 us vs 140 us), so it is launched plainly.
 // Every kernel executes griddepcontrol.launch_dependents, a no-op when the next launch is ordinary.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

@@ -104,3 +104,29 @@ def test_decode_over_compacted_cache(B):
     for l in range(tr.shape.L):
         TL.assert_decode_close(out[l].cpu().numpy(), qs[l], O.compact_rows(tr.keys(l), kept),
                                O.compact_rows(tr.values(l), kept), f"layer {l}")
+
+
+@pytest.mark.parametrize("G,d,h2o", [(1, 64, False), (4, 128, False), (5, 128, True), (8, 64, True)])
+@pytest.mark.parametrize("n", [1, 16, 17, 4099, 8190])
+def test_decode_stream_split(B, G, d, h2o, n):
+    """64 (layer, KV head) pairs of 8192-row caches: every warp streams a range of the list of all pairs' 16-key
+    blocks, so ranges begin and end inside pairs, in the last block's remainder, or hold no key at all.  Rows past n
+    hold NaN and must not be read into the result."""
+    import torch
+    rng = np.random.default_rng(7 * n + d + G)
+    Hkv, rows = 64, 8192
+    q, K, V = _bits(rng, (Hkv * G, d), 2.0), _bits(rng, (Hkv, n, d)), _bits(rng, (Hkv, n, d))
+    pad = lambda x: torch.cat([TL.bf16_dev(x), torch.full((Hkv, rows - n, d), float("nan"), dtype=torch.bfloat16,
+                                                          device="cuda")], 1)
+    Kd, Vd, st = [pad(K)], [pad(V)], B.new_status()
+    mass = [torch.zeros((Hkv, rows), dtype=torch.float32, device="cuda")]
+    out = B.stepkv_decode([TL.bf16_dev(q)], Kd, Vd, n, status=st)[0]
+    if h2o:
+        same = B.stepkv_decode_h2o([TL.bf16_dev(q)], Kd, Vd, n, mass, status=st)[0]
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    TL.assert_decode_close(out.cpu().numpy(), q, K, V, f"n {n}")
+    if h2o:
+        assert torch.equal(same, out)
+        TL.assert_close(mass[0][:, :n].cpu().numpy(), O.decode_attention_mass(q, K), "mass", floor=1e-30)
+        assert not mass[0][:, n:].any()
