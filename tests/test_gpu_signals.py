@@ -103,3 +103,22 @@ def test_signals_drive_the_fused_pass(B):
     out = O.compress(Ks, Qs, tr.step_id, tr.prot, tr.valid, og, orr, oo, tr.reuse, O.Params(), b.mode, b.num, b.den,
                      b.count)
     TL.check_select_outputs(g, out)
+
+
+@pytest.mark.parametrize("n_steps", [33, 34, 66])
+def test_step_signals_list_edges(B, n_steps):
+    """Lists of 0, 1, 63 and 64 cues over few ids (so fields of one step share cues and sets coincide), at step counts
+    around one round of a block's 32 warps."""
+    import torch
+    rng = np.random.default_rng(n_steps)
+    steps = [tuple(np.sort(rng.choice(80, rng.choice([0, 1, 63, 64]), replace=False)).astype(np.uint32) for _ in range(3))
+             for _ in range(n_steps)]
+    steps[n_steps // 2] = tuple(np.arange(2**32 - 64, 2**32, dtype=np.uint32) for _ in range(3))  # the largest ids
+    cues, cnt = _dev(steps)
+    st = B.new_status()
+    gain, red, obs_sim = B.stepkv_step_signals(cues, cnt, k0=0, status=st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    ref = O.step_signals([s[0] for s in steps], [s[1] for s in steps], [s[2] for s in steps], k0=0)
+    for got, want, name in zip((gain, red, obs_sim), ref, ("gain", "red", "obs_sim")):
+        assert np.allclose(got.cpu().numpy(), want, rtol=1e-6, atol=1e-7), name  # gain = 1 - sim near sim = 1
