@@ -364,6 +364,18 @@ def test_select_snapkv_pooling(B, pool, mode, T):
     TL.check_select_outputs(g, out)
 
 
+@pytest.mark.parametrize("rows, T", [(1, 255), (7, 256), (8, 257), (9, 513), (24, 4097)])
+@pytest.mark.parametrize("pool, mode", [(3, 0), (63, 0), (63, 1)])
+def test_select_pooling_row_batches(B, rows, T, pool, mode):
+    """Pooled rows are staged eight at a time over tiles of 256 tokens: row counts around a batch, lengths around a
+    tile, windows up to the widest (a halo on both sides, clipped at both ends)."""
+    tr = wl.custom(500 + T, L=1, Hq=2, Hkv=1, d=64, T=T, W=8, n_steps=4, budget=wl.Budget.ratio(1, 3))
+    sal = (np.random.default_rng(T + pool).random((rows, T)) ** 3).astype(np.float32)
+    g, out, st = _select_case(B, tr, B.Params(sal_pool=pool, sal_pool_mode=mode), sal)
+    assert st == 0
+    TL.check_select_outputs(g, out)
+
+
 @pytest.mark.parametrize("pool, mode, W, lse", [(7, 0, 64, False), (5, 1, 64, True), (3, 0, 128, False)])
 def test_compress_with_snapkv_pooling(B, pool, mode, W, lse):
     """The fused pass with a pooled token saliency: the saliency rows are written and pooled per
