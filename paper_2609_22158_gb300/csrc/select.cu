@@ -9,8 +9,8 @@
 //
 // GB300 design: the tokens live in shared memory (saliency, then the order-preserving 32-bit key of P,
 // and a 16-bit step id) -- in one 1024-thread CTA up to 2048 tokens, else in a cluster of 8 CTAs.
-// The exact B-th largest key is found by three radix passes (11/11/10 bits) over warp-aggregated
-// shared-memory histograms (summed across the cluster through distributed shared memory); retained
+// The exact B-th largest key is found by a linear bin of P and then digits of the key within that bin, over
+// shared-memory histograms whose sums meet through distributed shared memory; retained
 // slots are written in ascending order by warp ballot + prefix counts.  Per-step statistics use
 // integer atomics only (fixed-point sums), so every output is bit-reproducible run to run.
 #include <cooperative_groups.h>
@@ -26,11 +26,13 @@ namespace cg = cooperative_groups;
 namespace stepkv {
 
 // Two shapes of the same algorithm: one 1024-thread CTA for short trajectories (no cluster barriers),
-// else a cluster of 8 CTAs of 512 threads whose histograms and counts meet through distributed shared
-// memory.  Measured on GB300 at T = 32768: one CTA 78 us, 8-CTA cluster 31 us, 16-CTA cluster 35 us
-// (the token loops shrink with more SMs, the cluster barriers and DSMEM gathers grow).
+// else a cluster of 8 such CTAs whose histograms and counts meet through distributed shared memory.  One CTA up to 2048
+// tokens: at 4096 it is 2.9 us behind the cluster, at 8192 10 us.  1024 threads a CTA: a fused pass over T = 32768 takes
+// 257.7 us, 260.8 with 512 (the token loops are chains of short latencies, which more warps overlap and unrolling does
+// not: 258.1-258.6 us, the code is fetched cold).
 constexpr int kSelSingleMaxT = 2048;
 constexpr int kSelClusterCtas = 8;
+constexpr int kSelThreads = 1024;
 
 struct SelectArgs {
   const float* T_in;                  // token saliency as floats, or
@@ -53,22 +55,19 @@ struct SelectArgs {
   int32_t* status;
   // In-place compaction by hole filling (NULL plan: none).  The write pass also lays out the plan the move
   // kernel follows: plan[0] = number of holes H (slots below n_kept that are not retained), plan[1 + j] =
-  // the j-th hole in slot order; the j-th mover is kept_idx[n_kept - H + j].  Rows retained in place get
-  // their step id / position here; the move kernel writes those of the filled holes.
+  // the j-th hole in slot order; the j-th mover is kept_idx[n_kept - H + j].  All rows below n_kept get their own
+  // step id / position here; the move kernel overwrites those of the filled holes.
   int32_t* plan;
   const int32_t* pos_in;
   int32_t* step_id_out;
   int32_t* pos_out;
 };
 
-// Exchange block shared by the cluster (read remotely through DSMEM).
-struct SelShared {
-  float loc_max;
-  int loc_N;
-  int loc_err;
-  int loc_keep_base;   // protected + strictly-greater count
-  int loc_eq;          // ties at the threshold key
-  int pad[3];
+// One CTA's summary, pushed into every CTA of the cluster.
+struct SelSummary {
+  float max_T, min_T;  // over prunable tokens
+  int n;               // prunable tokens
+  int err;
 };
 
 // Several independent trajectories in one launch: cluster (or CTA) c selects for trajectory c, so the
@@ -89,83 +88,6 @@ __device__ __forceinline__ int warp_suffix_sum(int v, int lane) {
   return v;
 }
 
-template <int NT>
-__device__ __forceinline__ int block_reduce_sum_int(int v, int* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  int t = 0;
-  for (int w = 0; w < NT / 32; ++w) t += scratch[w];
-  return t;
-}
-
-template <int NT>
-__device__ __forceinline__ float block_reduce_max(float v, float* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if (lane == 0) scratch[warp] = v;
-  __syncthreads();
-  float t = -INFINITY;
-  for (int w = 0; w < NT / 32; ++w) t = fmaxf(t, scratch[w]);
-  return t;
-}
-
-// In-place exclusive prefix of arr[0..n) with starting value `init` (block-wide, fixed order).
-template <int NT>
-__device__ __forceinline__ void block_scan_array(int* arr, int n, int init, int* scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int per = (n + NT - 1) / NT;
-  const int lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
-  int mine = 0;
-  for (int i = lo; i < hi; ++i) mine += arr[i];
-  int x = mine;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  __syncthreads();
-  if (lane == 31) scratch[warp] = x;
-  __syncthreads();
-  int run = init + x - mine;
-  for (int w = 0; w < warp; ++w) run += scratch[w];
-  for (int i = lo; i < hi; ++i) {
-    const int c = arr[i];
-    arr[i] = run;
-    run += c;
-  }
-  __syncthreads();
-}
-
-// One step-statistics contribution per warp when the warp's (consecutive) tokens share one step, else
-// one per lane.  Integer atomics only: the totals do not depend on the order of arrival.
-__device__ __forceinline__ void step_stat_add(bool act, int sid, unsigned long long fx, uint32_t mx_bits, int32_t* cnt,
-                                              unsigned long long* sum, uint32_t* mx) {
-  const unsigned am = __ballot_sync(0xffffffffu, act);
-  if (!am) return;
-  const int lane = threadIdx.x & 31;
-  const int sid0 = __shfl_sync(0xffffffffu, sid, __ffs(am) - 1);
-  if (__all_sync(0xffffffffu, !act || sid == sid0)) {
-    unsigned long long v = act ? fx : 0ull;
-    uint32_t m = act ? mx_bits : 0u;
-    for (int o = 16; o > 0; o >>= 1) {
-      v += __shfl_xor_sync(0xffffffffu, v, o);
-      m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    }
-    if (lane == 0) {
-      atomicAdd(&cnt[sid0], __popc(am));
-      if (sum) atomicAdd(&sum[sid0], v);
-      if (mx) atomicMax(&mx[sid0], m);
-    }
-  } else if (act) {
-    atomicAdd(&cnt[sid], 1);
-    if (sum) atomicAdd(&sum[sid], fx);
-    if (mx) atomicMax(&mx[sid], mx_bits);
-  }
-}
-
 // Warp-wide flush of per-lane step statistics (lane: `act`, its step `sid`, count, fixed-point sum,
 // max bits): one set of atomics per warp when every active lane holds the same step, else one per
 // lane.  Integer atomics only, so the totals do not depend on the order of arrival.
@@ -177,13 +99,12 @@ __device__ __forceinline__ void step_stat_flush(bool act, int sid, int cnt_v, un
   const int lane = threadIdx.x & 31;
   const int sid0 = __shfl_sync(0xffffffffu, sid, __ffs(am) - 1);
   if (__all_sync(0xffffffffu, !act || sid == sid0)) {
-    int c = act ? cnt_v : 0;
+    const int c = __reduce_add_sync(0xffffffffu, act ? cnt_v : 0);
     unsigned long long v = act ? sum_v : 0ull;
-    uint32_t m = act ? max_v : 0u;
-    for (int o = 16; o > 0; o >>= 1) {
-      c += __shfl_xor_sync(0xffffffffu, c, o);
-      if (sum) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (mx) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const uint32_t m = mx ? __reduce_max_sync(0xffffffffu, act ? max_v : 0u) : 0u;
+    if (sum) {
+#pragma unroll 1
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     }
     if (lane == 0) {
       atomicAdd(&cnt[sid0], c);
@@ -197,17 +118,19 @@ __device__ __forceinline__ void step_stat_flush(bool act, int sid, int cnt_v, un
   }
 }
 
-__device__ __forceinline__ float step_utility(const SelectArgs& a, int k, int t_last, float* c_out) {
-  const stepkv_params_t& p = a.prm;
-  const float r = a.steps.valid[k] + a.steps.gain[k] - p.lambda * a.steps.red[k];  // Eq. 2
+__device__ __forceinline__ float step_reuse(const SelectArgs& a, int k, int t_last) {
   float c = 0.f;                                                                     // Alg. 1: c_t = 0
   if (k != t_last) {
     c = a.steps.reuse_in[k];
-    if (a.steps.obs_sim) c += fminf(1.f, p.eta * a.steps.obs_sim[k]);              // Eq. 3
+    if (a.steps.obs_sim) c += fminf(1.f, a.prm.eta * a.steps.obs_sim[k]);          // Eq. 3
   }
-  *c_out = c;
+  return c;
+}
+__device__ __forceinline__ float step_utility(const SelectArgs& a, int k, int t_last) {
+  const stepkv_params_t& p = a.prm;
+  const float r = a.steps.valid[k] + a.steps.gain[k] - p.lambda * a.steps.red[k];  // Eq. 2
   const float rc = fminf(fmaxf(r, p.r_min), p.r_max);
-  return fminf(fmaxf(p.w_r * rc + p.w_c * log1pf(c), 0.f), p.s_max);               // Eq. 4
+  return fminf(fmaxf(p.w_r * rc + p.w_c * log1pf(step_reuse(a, k, t_last)), 0.f), p.s_max);  // Eq. 4
 }
 
 template <int NC>
@@ -227,173 +150,189 @@ struct ClusterOps<1> {
   __device__ P* peer(P* p, int) { return p; }
 };
 
-template <int NC, int NT>
+// What bounds a selection is latency: barriers, distributed-shared-memory round trips, and code that runs once per
+// launch and is fetched cold (so loops stay rolled).  There are as few of each as
+// the result allows:
+//  - the first digit is a linear bin of the priority between its bounds (the corners of alpha T^ + beta S over the
+//    extreme T^ and S), so the bins spread over the values the trajectory has; the keys of the threshold's bin span about
+//    BITS bits, and one more pass over the key's offset within the bin ranks them exactly (further passes where the bin
+//    reaches down to where floats are dense).  Fixed digits of the key took three passes, the first of which only told
+//    a few exponents apart;
+//  - every exchange is a push into the other CTAs' shared memory before a cluster barrier, so only the 32 fine counts
+//    of each digit are fetched after one;
+//  - a CTA's output offset comes out of the same counts (those of the CTAs before it above each digit), so no
+//    barrier is spent on it; the barrier that lets CTAs exit is split around the writes.
+// Against three fixed digits with a gather after every barrier: a fused pass over T = 32768 263.5 -> 256.0 us, over
+// T = 65536 864.6 -> 856, T = 2048 35.6 -> 31.9, an in-place boundary 102.1 -> 96.9, a selection alone with all outputs
+// 26.6 -> 22.6.
+// BITS: 13, or 11 where the tokens leave no room for 2 x 8192 bins.
+template <int NC, int NT, int BITS>
 __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ SelectBatch batch) {
   const SelectArgs& a = batch.t[blockIdx.x / NC];
   constexpr int NW = NT / 32;
-  constexpr int UNROLL = NT >= 1024 ? 4 : 8;
+  constexpr int U = 4;  // tokens of a thread in flight
+  constexpr int kBins = 1 << BITS, kCoarse = kBins / 32;
   ClusterOps<NC> cl;
   const int rank = cl.rank();
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  // layout: [chunk] float/uint32 keys | [chunk] u16 step id (0xFFFF = protected) | 2 x 2048 int hist |
-  //         SelShared (own) | SelShared[NC] (gathered) | scratch[64] | coarse[2][NC][64] | S_k (when s_in_smem)
-  uint32_t* sKey = reinterpret_cast<uint32_t*>(smem_raw);
-  float* sT = reinterpret_cast<float*>(smem_raw);
-  uint16_t* sSid = reinterpret_cast<uint16_t*>(smem_raw + (size_t)a.chunk * 4);
-  int* hist = reinterpret_cast<int*>(smem_raw + (((size_t)a.chunk * 6 + 15) & ~size_t(15)));
-  SelShared* ex = reinterpret_cast<SelShared*>(hist + 2 * 2048);
-  SelShared* all = ex + 1;
-  int* scratch = reinterpret_cast<int*>(all + NC);  // 64 ints
-  int* bcast = scratch + 48;                        // radix decision
-  int* allc = scratch + 64;                         // [2 passes][NC ranks][64] every CTA's coarse counts
-  float* sS = reinterpret_cast<float*>(allc + 2 * NC * 64);
+  // layout: [2][kBins] int histograms | [2][NC][kCoarse] every CTA's coarse counts | [chunk] T, then the ordered key of
+  // P | [chunk] u16 step id (0xFFFF = protected) | S_k (when s_in_smem).  A token's entries are touched by one thread only.
+  int* hist = reinterpret_cast<int*>(smem_raw);
+  int* coarse = hist + 2 * kBins;
+  uint32_t* sKey = reinterpret_cast<uint32_t*>(coarse + 2 * NC * kCoarse);
+  float* sT = reinterpret_cast<float*>(sKey);
+  uint16_t* sSid = reinterpret_cast<uint16_t*>(sKey + a.chunk);
+  float* sS = reinterpret_cast<float*>(sSid + a.chunk);
+  __shared__ SelSummary all[NC];
+  __shared__ float w_max[NW], w_min[NW], s_lo[NW], s_hi[NW];
+  __shared__ int w_n[NW], w_err[NW], w_strict[NW], w_eq[NW], bcast[4];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int T = a.T;
-  const int n_steps = a.steps.n_steps;
-  const int t_last = n_steps - 1;
+  const int T = a.T, n_steps = a.steps.n_steps, t_last = n_steps - 1;
   const int base = rank * a.chunk;
   const int len = max(0, min(a.chunk, T - base));
-  const bool s_in_smem = a.s_in_smem != 0;
-  // per-step statistics are outputs only (they do not enter P): skip them when none is requested
   const bool want_stats = a.out.step_count || a.out.step_sal_sum || a.out.step_sal_max;
   const bool want_kept = a.out.step_kept != nullptr;
+  const bool s_in_smem = a.s_in_smem != 0;
+  // warp w owns the consecutive slots [s0, s1) of this CTA, lanes take consecutive slots
+  const int seg = ((len + NW - 1) / NW + 31) & ~31;
+  const int s0 = min(len, warp * seg), s1 = min(len, s0 + seg);
+  const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
 
-  // Launched with programmatic dependent launch: everything up to pdl_wait() reads only the call's
-  // inputs (step signals, step ids, mask) and writes only this kernel's workspace and outputs, so it
-  // may overlap the tail of the kernel that produces the token saliency.
+  // Launched with programmatic dependent launch: everything up to pdl_wait() reads only the call's inputs and writes
+  // only this kernel's workspace and outputs, so it may overlap the tail of the kernel that produces the saliency.
   pdl_launch_dependents();
-
-  // ---- Phase 1+2 of Algorithm 1 (Eqs. 2-4).  With few steps every CTA keeps all S_k in shared memory
-  // (CTA 0 publishes them); otherwise the steps are split over the CTAs through global memory.
-  if (s_in_smem) {
-    for (int k = tid; k < n_steps; k += NT) {
-      float c;
-      const float sk = step_utility(a, k, t_last, &c);
-      sS[k] = sk;
-      if (rank == 0) {
-        a.S[k] = sk;
-        if (a.out.step_util) a.out.step_util[k] = sk;
-        // reuse_out may alias reuse_in, which every CTA reads here: written after barrier (A)
-      }
-    }
-  } else {
-    for (int k = rank * NT + tid; k < n_steps; k += NC * NT) {
-      float c;
-      const float sk = step_utility(a, k, t_last, &c);
-      a.S[k] = sk;
-      if (a.out.step_util) a.out.step_util[k] = sk;
-      if (a.steps.reuse_out) a.steps.reuse_out[k] = c;
-    }
-  }
-  if (a.plan && rank == 0 && tid == 0) a.plan[0] = 0;  // hole count, summed after barrier (B)
-  for (int k = rank * NT + tid; k < n_steps; k += NC * NT) {
-    a.acc_cnt[k] = 0;
-    a.acc_sum[k] = 0ull;
-    a.acc_max[k] = 0u;
-    a.acc_kept[k] = 0;
-  }
-
-  // ---- this CTA's tokens: step ids / protection flags (inputs), then, once the producing kernel has
-  // finished, token saliency T_i (loads batched)
-  float lmax = -INFINITY;
   int lN = 0, lerr = 0;
-  for (int i0 = 0; i0 < len; i0 += NT * UNROLL) {
-    uint8_t pv[UNROLL];
-    int sv[UNROLL];
+#pragma unroll 1
+  for (int i0 = s0 + lane; i0 < s1; i0 += 32 * U) {
+    uint8_t pv[U];
+    int sv[U];
 #pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const int i = i0 + u * NT + tid;
-      if (i < len) {
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u;
+      if (i < s1) {
         pv[u] = __ldg(&a.prot[base + i]);
         sv[u] = __ldg(&a.step_id[base + i]);
       }
     }
 #pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const int i = i0 + u * NT + tid;
-      if (i < len) {
-        if (!pv[u]) {
-          ++lN;
-          const bool bad = sv[u] < 0 || sv[u] >= n_steps;
-          if (bad) lerr = 1;
-          sSid[i] = bad ? 0 : (uint16_t)sv[u];
-        } else {
-          sSid[i] = 0xFFFFu;
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u;
+      if (i < s1) {
+        const bool bad = !pv[u] && (sv[u] < 0 || sv[u] >= n_steps);
+        lN += !pv[u];
+        lerr |= bad;
+        sSid[i] = pv[u] ? (uint16_t)0xFFFFu : (uint16_t)(bad ? 0 : sv[u]);
+      }
+    }
+  }
+#pragma unroll 1
+  for (int i = tid; i < 2 * kBins / 4; i += NT) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+  // Phases 1 and 2 of Algorithm 1 (Eqs. 2-4).  Every CTA computes all S_k, for their bounds and, where they fit, into
+  // shared memory; CTA 0 publishes them.
+  float b_lo = INFINITY, b_hi = -INFINITY;  // bounds of beta S_k
+#pragma unroll 1
+  for (int k = tid; k < n_steps; k += NT) {
+    const float sk = step_utility(a, k, t_last);
+    if (s_in_smem) sS[k] = sk;
+    b_lo = fminf(b_lo, a.prm.beta * sk);
+    b_hi = fmaxf(b_hi, a.prm.beta * sk);
+    if (rank == 0) {
+      a.S[k] = sk;
+      if (a.out.step_util) a.out.step_util[k] = sk;  // reuse_out may alias reuse_in: written after the barrier
+    }
+    if (k % NC == rank) {
+      a.acc_cnt[k] = 0;
+      a.acc_sum[k] = 0ull;
+      a.acc_max[k] = 0u;
+      a.acc_kept[k] = 0;
+    }
+  }
+  if (a.plan && rank == 0 && tid == 0) a.plan[0] = 0;  // hole count
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    b_lo = fminf(b_lo, __shfl_xor_sync(full, b_lo, o));
+    b_hi = fmaxf(b_hi, __shfl_xor_sync(full, b_hi, o));
+  }
+  lN = __reduce_add_sync(full, lN);
+  lerr = __any_sync(full, lerr);
+  if (lane == 0) {
+    s_lo[warp] = b_lo;
+    s_hi[warp] = b_hi;
+    w_n[warp] = lN;
+    w_err[warp] = lerr;
+  }
+  pdl_wait();  // t_acc / T_in come from the preceding kernel
+  float lmax = -INFINITY, lmin = INFINITY;
+#pragma unroll 1
+  for (int i0 = s0 + lane; i0 < s1; i0 += 32 * U) {
+    float tv[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u;
+      if (i < s1) tv[u] = a.t_acc ? __ull2float_rn(__ldcg(&a.t_acc[base + i])) * a.acc_to_T : __ldcg(&a.T_in[base + i]);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + 32 * u;
+      if (i < s1) {
+        sT[i] = tv[u];
+        if (sSid[i] != 0xFFFFu) {
+          lmax = fmaxf(lmax, tv[u]);
+          lmin = fminf(lmin, tv[u]);
         }
       }
     }
   }
-  pdl_wait();  // t_acc / T_in come from the preceding kernel
-  for (int i0 = 0; i0 < len; i0 += NT * UNROLL) {
-    float tv[UNROLL];
 #pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const int i = i0 + u * NT + tid;
-      if (i < len) {
-        const int gi = base + i;
-        tv[u] = a.t_acc ? __ull2float_rn(__ldcg(&a.t_acc[gi])) * a.acc_to_T : __ldcg(&a.T_in[gi]);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < UNROLL; ++u) {
-      const int i = i0 + u * NT + tid;
-      if (i < len) {
-        sT[i] = tv[u];
-        if (sSid[i] != 0xFFFFu) lmax = fmaxf(lmax, tv[u]);  // this thread wrote sSid[i] above
-      }
-    }
+  for (int o = 16; o > 0; o >>= 1) {
+    lmax = fmaxf(lmax, __shfl_xor_sync(full, lmax, o));
+    lmin = fminf(lmin, __shfl_xor_sync(full, lmin, o));
   }
-  {
-    // one block reduction for (max T, prunable count, error flag); the histogram area is free here
-    for (int o = 16; o > 0; o >>= 1) {
-      lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-      lN += __shfl_xor_sync(0xffffffffu, lN, o);
-      lerr |= __shfl_xor_sync(0xffffffffu, lerr, o);
-    }
-    float* red_max = reinterpret_cast<float*>(hist);
-    int* red_n = hist + NW;
-    int* red_e = hist + 2 * NW;
-    if (lane == 0) {
-      red_max[warp] = lmax;
-      red_n[warp] = lN;
-      red_e[warp] = lerr;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      float bm = -INFINITY;
-      int bn = 0, be = 0;
-      for (int w = 0; w < NW; ++w) {
-        bm = fmaxf(bm, red_max[w]);
-        bn += red_n[w];
-        be |= red_e[w];
-      }
-      ex->loc_max = bm;
-      ex->loc_N = bn;
-      ex->loc_err = be;
-    }
-  }
-  cl.sync();  // (A) S_k, zeroed accumulators and per-CTA summaries visible to every CTA
-  if (s_in_smem && rank == 0 && a.steps.reuse_out) {
-    for (int k = tid; k < n_steps; k += NT) {
-      float c;
-      step_utility(a, k, t_last, &c);
-      a.steps.reuse_out[k] = c;
-    }
-  }
-  if (tid < NC) {
-    const int4* rex = reinterpret_cast<const int4*>(cl.peer(ex, tid));
-    const int4 v0 = rex[0], v1 = rex[1];
-    reinterpret_cast<int4*>(&all[tid])[0] = v0;
-    reinterpret_cast<int4*>(&all[tid])[1] = v1;
+  if (lane == 0) {
+    w_max[warp] = lmax;
+    w_min[warp] = lmin;
   }
   __syncthreads();
-  float gmax = -INFINITY;
-  int N = 0, err = 0;
+  if (warp == 0) {
+    float m = lane < NW ? w_max[lane] : -INFINITY, mi = lane < NW ? w_min[lane] : INFINITY;
+    b_lo = lane < NW ? s_lo[lane] : INFINITY;
+    b_hi = lane < NW ? s_hi[lane] : -INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      m = fmaxf(m, __shfl_xor_sync(full, m, o));
+      mi = fminf(mi, __shfl_xor_sync(full, mi, o));
+      b_lo = fminf(b_lo, __shfl_xor_sync(full, b_lo, o));
+      b_hi = fmaxf(b_hi, __shfl_xor_sync(full, b_hi, o));
+    }
+    const int n = __reduce_add_sync(full, lane < NW ? w_n[lane] : 0);
+    const int err = __reduce_or_sync(full, lane < NW ? w_err[lane] : 0);
+    if (lane < NC) {
+      SelSummary* dst = cl.peer(&all[rank], lane);
+      dst->max_T = m;
+      dst->min_T = mi;
+      dst->n = n;
+      dst->err = err;
+    }
+    if (lane == 0) {
+      s_lo[0] = b_lo;
+      s_hi[0] = b_hi;
+    }
+  }
+  cl.sync();  // every CTA's summary is here; S_k, histograms and zeroed accumulators are ready
+  if (rank == 0 && a.steps.reuse_out) {
+#pragma unroll 1
+    for (int k = tid; k < n_steps; k += NT) a.steps.reuse_out[k] = step_reuse(a, k, t_last);
+  }
+  float gmax = -INFINITY, gmin = INFINITY;
+  int N = 0, err = 0, n_pre = 0;  // n_pre: prunable tokens of the CTAs before this one
+#pragma unroll
   for (int r = 0; r < NC; ++r) {
-    gmax = fmaxf(gmax, all[r].loc_max);
-    N += all[r].loc_N;
-    err += all[r].loc_err;
+    gmax = fmaxf(gmax, all[r].max_T);
+    gmin = fminf(gmin, all[r].min_T);
+    if (r < rank) n_pre += all[r].n;
+    N += all[r].n;
+    err |= all[r].err;
   }
   if (err) {
     if (rank == 0 && tid == 0) {
@@ -401,7 +340,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
       *a.out.n_kept = 0;
       if (a.out.n_budget) { a.out.n_budget[0] = N; a.out.n_budget[1] = 0; }
     }
-    cl.sync();
+    if (NC > 1) cl.sync();
     return;
   }
   // ---- budget (Eq. 1): B = max(1, floor(num N / den)) or a count, then |K| = min(B, N)
@@ -413,41 +352,54 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
       B = a.budget.count;
     B = min(B, N);
   }
+  const int total_kept = T - N + B;
+  const bool overflow = total_kept > a.out.kept_cap;
+  // In place: the step ids and positions of the rows below total_kept, holes included (the move kernel overwrites
+  // those), copied by warps w0 .. of every CTA, a CTA's own slots.
+  auto copy_metadata = [&](int w0) {
+    if (!a.plan || overflow) return;
+    for (int i = (warp - w0) * 32 + lane; i < len && base + i < total_kept; i += (NW - w0) * 32) {
+      const int gi = base + i;
+      const int sid = a.step_id_out ? __ldg(&a.step_id[gi]) : 0, pos = a.pos_in ? __ldg(&a.pos_in[gi]) : gi;
+      if (a.step_id_out) a.step_id_out[gi] = sid;
+      if (a.pos_out) a.pos_out[gi] = pos;
+    }
+  };
   const bool norm = a.prm.sal_norm == STEPKV_NORM_MAX && gmax > 0.f && N > 0;
   const float inv_max = norm ? 1.0f / gmax : 1.0f;
   // fixed-point scale for per-step sums of normalised saliency: values <= vmax, at most N terms
   const float vmax = norm ? 1.0f : fmaxf(gmax, 1e-30f);
-  int e_max;
-  frexpf(vmax, &e_max);                       // vmax < 2^e_max
-  const int log2N = 32 - __clz(max(N, 1));    // N < 2^log2N
+  const int e_max = (int)(__float_as_uint(vmax) >> 23) - 126;  // vmax < 2^e_max (vmax is normal and positive)
+  const int log2N = 32 - __clz(max(N, 1));            // N < 2^log2N
   const int fx_shift = min(62 - log2N - e_max, 126);  // every partial sum < 2^62
+
+  // ---- priorities (Eq. 5) and their bounds; bins of the first digit
+  const float t_lo = gmin * inv_max, t_hi = gmax * inv_max;
+  const float P_lo = fminf(fmaf(a.prm.alpha, t_lo, s_lo[0]), fmaf(a.prm.alpha, t_hi, s_lo[0]));
+  const float P_hi = fmaxf(fmaf(a.prm.alpha, t_lo, s_hi[0]), fmaf(a.prm.alpha, t_hi, s_hi[0]));
+  const float scale = P_hi > P_lo ? 0.999999f * (float)kBins / (P_hi - P_lo) : 0.f;
+  auto first_bin = [&](uint32_t key) {  // monotone in the priority
+    return min(max((int)((ordered_to_float(key) - P_lo) * scale), 0), kBins - 1);
+  };
   const float* Sk = s_in_smem ? sS : a.S;
-
-  // Warp w owns the consecutive slots [w*seg, (w+1)*seg) of this CTA in the passes that need slot order
-  // or per-step runs (keys and statistics, counts, ordered write); lanes take consecutive slots.
-  const int seg = ((len + NW - 1) / NW + 31) & ~31;
-  const int s0 = min(len, warp * seg), s1 = min(len, s0 + seg);
-
-  // ---- priorities (Eq. 5), ordered keys and per-step statistics.  A lane accumulates its tokens'
-  // statistics while their step does not change (slots of a step are mostly contiguous) and flushes
-  // with integer atomics; T_hat is read before its shared-memory slot is overwritten by the key.
   {
+    // A lane accumulates its tokens' statistics while their step does not change (slots of a step are mostly
+    // contiguous) and flushes with integer atomics.
     int run_sid = -1, run_c = 0;
     unsigned long long run_s = 0ull;
     uint32_t run_m = 0u;
-    for (int i0 = s0; i0 < s1; i0 += 32) {
-      const int i = i0 + lane;
-      if (i >= s1) break;
+#pragma unroll 1
+    for (int i = s0 + lane; i < s1; i += 32) {
       const int gi = base + i;
-      const float th = sT[i] * inv_max;
+      const float x = sT[i] * inv_max;
       const int sid = sSid[i];
       uint32_t key = 0u;
+      float P = -INFINITY;
       if (sid != 0xFFFF) {
-        const float P = fmaf(a.prm.alpha, th, a.prm.beta * Sk[sid]);
+        P = fmaf(a.prm.alpha, x, a.prm.beta * Sk[sid]);
         key = float_to_ordered(P);
-        if (a.out.priority) a.out.priority[gi] = P;
         if (want_stats) {
-          const float thc = fmaxf(th, 0.f);
+          const float xc = fmaxf(x, 0.f);
           if (sid != run_sid) {
             if (run_c) {
               atomicAdd(&a.acc_cnt[run_sid], run_c);
@@ -460,195 +412,226 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
             run_m = 0u;
           }
           ++run_c;
-          run_s += to_fixed(thc, fx_shift);
-          run_m = max(run_m, __float_as_uint(thc));
+          run_s += to_fixed(xc, fx_shift);
+          run_m = max(run_m, __float_as_uint(xc));
         }
-      } else if (a.out.priority) {
-        a.out.priority[gi] = -INFINITY;
       }
-      if (a.out.token_sal) a.out.token_sal[gi] = th;
+      if (a.out.priority) a.out.priority[gi] = P;
+      if (a.out.token_sal) a.out.token_sal[gi] = x;
       sKey[i] = key;
     }
-    step_stat_flush(run_c > 0, run_sid, run_c, run_s, run_m, a.acc_cnt, a.acc_sum, a.acc_max);
+    if (want_stats) step_stat_flush(run_c > 0, run_sid, run_c, run_s, run_m, a.acc_cnt, a.acc_sum, a.acc_max);
   }
-  __syncthreads();
 
-  // ---- exact radix select of the B-th largest key among prunable tokens
-  uint32_t kth = 0u;
+  // ---- exact B-th largest key among the prunable tokens
+  uint32_t kth = 0u;  // B == N: every prunable token's key is above 0
   int need_eq = 0;
+  int strict_pre = n_pre, eq_pre = 0;  // tokens above / at the threshold in the CTAs before this one
   if (B == 0) {
     kth = 0xFFFFFFFFu;
+    strict_pre = 0;
   } else if (B < N) {
-    uint32_t prefix = 0u, mask = 0u;
-    int remaining = B;
-    for (int pass = 0; pass < 3; ++pass) {
-      int* h = hist + (pass & 1) * 2048;
-      const int nbits = pass < 2 ? 11 : 10;
-      const int sh = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-      const int nb = 1 << nbits;
-      for (int b = tid; b < nb; b += NT) h[b] = 0;
-      __syncthreads();
-      // keys of one step share their leading bits, so many lanes hit the same bin: aggregate per warp
-      for (int i0 = 0; i0 < len; i0 += NT) {
-        const int i = i0 + tid;
-        const uint32_t k = i < len ? sKey[i] : 0u;
-        const bool hit = i < len && sSid[i] != 0xFFFF && (k & mask) == prefix;
-        if (__ballot_sync(0xffffffffu, hit) == 0u) continue;  // after the first pass most keys miss the prefix
-        const int bin = hit ? (int)((k >> sh) & (nb - 1)) : -1;
-        const unsigned peers = __match_any_sync(0xffffffffu, bin);
-        if (hit && (__ffs(peers) - 1) == lane) atomicAdd(&h[bin], __popc(peers));
+    strict_pre = 0;
+    int remaining = B, star = -1;      // star: the threshold's first bin
+    uint32_t k_lo = 0u, prefix = 0u;   // later passes: keys of that bin as offsets from k_lo, `left` bits undecided
+    int left = 0;
+#pragma unroll 1
+    for (int pass = 0;; ++pass) {
+      int* h = hist + (pass & 1) * kBins;
+      int* ac = coarse + (pass & 1) * NC * kCoarse;
+      const int bits = pass == 0 ? BITS : min(BITS, left), sh = left - bits;  // of the key offset (later passes)
+      const int n_coarse = pass == 0 ? kCoarse : max(1, (1 << bits) >> 5);
+      if (pass >= 2) {  // the buffers were zeroed for two passes
+#pragma unroll 1
+        for (int i = tid; i < kBins / 4; i += NT) reinterpret_cast<int4*>(h)[i] = make_int4(0, 0, 0, 0);
+        __syncthreads();
+      }
+#pragma unroll 1
+      for (int i0 = s0; i0 < s1; i0 += 32) {
+        const int i = i0 + lane;
+        bool hit = i < s1 && sSid[i] != 0xFFFF;
+        int bin = 0;
+        if (hit) {
+          const uint32_t key = sKey[i];
+          bin = first_bin(key);
+          if (pass > 0) {
+            const uint32_t off = key - k_lo;
+            hit = bin == star && (left >= 32 || (off >> left) == prefix);
+            bin = (int)((off >> sh) & ((1u << bits) - 1u));
+          }
+        }
+        const unsigned hm = __ballot_sync(full, hit);
+        if (hm == 0u) continue;
+        // tokens of one warp mostly fall into bins of their own; equal priorities share one addition
+        const int b0 = __shfl_sync(full, bin, __ffs(hm) - 1);
+        if (__all_sync(full, !hit || bin == b0)) {
+          if (lane == 0) atomicAdd(&h[b0], __popc(hm));
+        } else if (hit) {
+          atomicAdd(&h[bin], 1);
+        }
       }
       __syncthreads();
-      // this CTA's coarse counts: sums of 32 consecutive bins (64 coarse bins for 11 bits, 32 for 10),
-      // pushed into every CTA's table before the barrier (lane r stores into rank r), so the coarse step
-      // below reads them from its own shared memory
-      int* ac = allc + (pass & 1) * NC * 64;
-      const int ncoarse = nb >> 5;
-      for (int c = warp; c < ncoarse; c += NW) {
-        int v = h[c * 32 + lane];
+      // sums of 32 consecutive bins, NW warps over the coarse bins, pushed into every CTA (lane i holds sum i)
+      constexpr int kPerWarp = kCoarse / NW;
+      if (warp * kPerWarp < n_coarse) {
+        int mine = 0;
+#pragma unroll 4
+        for (int i = 0; i < kPerWarp; ++i) {
+          const int v = __reduce_add_sync(full, h[(warp * kPerWarp + i) * 32 + lane]);
+          if (lane == i) mine = v;
+        }
+        if (lane < kPerWarp) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane < NC) cl.peer(ac, lane)[rank * 64 + c] = v;
+          for (int r = 0; r < NC; ++r) cl.peer(ac, r)[rank * kCoarse + warp * kPerWarp + lane] = mine;
+        }
       }
       cl.sync();  // every CTA's histogram and coarse counts of this pass are complete
       if (warp == 0) {
-        // The digit in two small cluster-wide steps (keys in descending order): first the coarse bin that
-        // holds the remaining-th largest key, then the bin within it.  Lane l holds coarse bins l and
-        // 32 + l, then fine bin 32 * c* + l.
-        int clo = 0, chi = 0;
+        // The digit in two steps (keys in descending order): the coarse bin that holds the remaining-th largest key
+        // (lane l: coarse bins 8 l .. 8 l + 7), then the bin within it (lane l: fine bin l).
+        constexpr int PL = kCoarse / 32;
+        int cnt[PL];
+#pragma unroll
+        for (int i = 0; i < PL; ++i) cnt[i] = 0;
+        if (lane * PL < n_coarse) {
+#pragma unroll
+          for (int r = 0; r < NC; ++r) {
+#pragma unroll
+            for (int i = 0; i < PL; i += 4) {
+              const int4 v = *reinterpret_cast<const int4*>(&ac[r * kCoarse + lane * PL + i]);
+              const int w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+              for (int x = 0; x < 4; ++x) cnt[i + x] += lane * PL + i + x < n_coarse ? w[x] : 0;
+            }
+          }
+        }
+        int mine = 0;
+#pragma unroll
+        for (int i = 0; i < PL; ++i) mine += cnt[i];
+        int above = warp_suffix_sum(mine, lane) - mine;  // keys in the coarse bins of the lanes after this one
+        int cs = -1, above_c = 0;
+#pragma unroll
+        for (int i = PL - 1; i >= 0; --i) {
+          if (cs < 0 && above < remaining && remaining <= above + cnt[i]) {
+            cs = lane * PL + i;
+            above_c = above;
+          }
+          above += cnt[i];
+        }
+        const unsigned mc = __ballot_sync(full, cs >= 0);
+        const int src = mc ? __ffs(mc) - 1 : 0;
+        const int cstar = max(0, __shfl_sync(full, cs, src));
+        above_c = __shfl_sync(full, above_c, src);
+        int f = 0, f_p = 0;
 #pragma unroll
         for (int r = 0; r < NC; ++r) {
-          clo += ac[r * 64 + lane];
-          if (ncoarse > 32) chi += ac[r * 64 + 32 + lane];
+          const int v = cl.peer(h, r)[cstar * 32 + lane];
+          f += v;
+          if (r < rank) f_p += v;
         }
-        const int shi = warp_suffix_sum(chi, lane);                                    // keys in bins >= 32 + l
-        const int slo = warp_suffix_sum(clo, lane) + __shfl_sync(0xffffffffu, shi, 0);  // keys in bins >= l
-        const unsigned mhi = __ballot_sync(0xffffffffu, shi - chi < remaining && remaining <= shi);
-        const unsigned mlo = __ballot_sync(0xffffffffu, slo - clo < remaining && remaining <= slo);
-        const int lhi = __ffs(mhi) - 1, llo = __ffs(mlo) - 1;
-        const int above_hi = __shfl_sync(0xffffffffu, shi - chi, lhi < 0 ? 0 : lhi);
-        const int above_lo = __shfl_sync(0xffffffffu, slo - clo, llo < 0 ? 0 : llo);
-        bool found = mhi != 0 || mlo != 0;
-        const int cstar = mhi ? 32 + lhi : (mlo ? llo : 0);
-        const int above_c = mhi ? above_hi : (mlo ? above_lo : 0);
-        int f = 0;
+        int pre = 0;  // in the coarse bins above c*, of the CTAs before this one
+#pragma unroll 1
+        for (int i = cstar + 1 + lane; i < n_coarse; i += 32)
 #pragma unroll
-        for (int r = 0; r < NC; ++r) f += cl.peer(h, r)[cstar * 32 + lane];
+          for (int r = 0; r < NC; ++r)
+            if (r < rank) pre += ac[r * kCoarse + i];
         const int sf = warp_suffix_sum(f, lane);
-        const unsigned mf = __ballot_sync(0xffffffffu, above_c + sf - f < remaining && remaining <= above_c + sf);
-        const int lf = __ffs(mf) - 1;
-        found = found && mf != 0;
-        const int above_f = __shfl_sync(0xffffffffu, above_c + sf - f, lf < 0 ? 0 : lf);
-        if (lane == 0) {
+        const unsigned mf = __ballot_sync(full, above_c + sf - f < remaining && remaining <= above_c + sf);
+        const int lf = mf ? __ffs(mf) - 1 : 0;
+        const int above_f = __shfl_sync(full, above_c + sf - f, lf);
+        pre = __reduce_add_sync(full, pre + (lane > lf ? f_p : 0));
+        if (lane == lf) {
           // the counts always hold the remaining-th key; the guard only keeps every index in range
+          const bool found = mc != 0 && mf != 0;
           if (!found) record_status(a.status, STEPKV_EDATA);
           bcast[0] = found ? cstar * 32 + lf : 0;
           bcast[1] = found ? above_f : 0;
+          bcast[2] = pre;
+          bcast[3] = f_p;
         }
+      } else if (pass == 0) {
+        copy_metadata(1);  // while the first warp searches
       }
       __syncthreads();
-      const int bstar = bcast[0];
+      const int digit = bcast[0];
       remaining -= bcast[1];
-      prefix |= (uint32_t)bstar << sh;
-      mask |= (uint32_t)(nb - 1) << sh;
-      __syncthreads();
+      strict_pre += bcast[2];
+      eq_pre = bcast[3];
+      if (pass == 0) {
+        // the keys of the bin lie within its bounds, widened by its rounding and two keys
+        star = digit;
+        uint32_t k_hi = float_to_ordered(P_hi);
+        k_lo = float_to_ordered(P_lo);
+        const float w = 1.0f / scale;
+        if (scale > 0.f && w > 0.f) {
+          const uint32_t lo = float_to_ordered(P_lo + ((float)star - 0.02f) * w) - 2u;
+          const uint32_t hi = float_to_ordered(P_lo + ((float)star + 1.02f) * w) + 2u;
+          if (star > 0) k_lo = max(k_lo, lo);
+          if (star < kBins - 1) k_hi = min(k_hi, hi);
+        }
+        left = 32 - __clz((int)(k_hi - k_lo));  // 0: one value
+      } else {
+        prefix = (bits < 32 ? prefix << bits : 0u) | (uint32_t)digit;
+        left = sh;
+      }
+      if (left == 0) break;
     }
-    kth = prefix;
+    kth = k_lo + prefix;
     need_eq = remaining;
   }
-  // B == N: kth = 0 keeps every prunable token (all prunable keys are > 0)
+  if (B == 0 || B == N) copy_metadata(0);
+  if (NC > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");  // no more reads of other CTAs' memory
 
-  // ---- counts per warp segment: kept for sure (protected or strictly above the threshold) and ties
-  int strict_w = 0, eq_w = 0;  // warp-uniform
-  for (int i0 = s0; i0 < s1; i0 += 32) {
-    const int i = i0 + lane;
-    const bool in = i < s1;
-    const uint32_t k = in ? sKey[i] : 0u;
-    const bool pr = in && sSid[i] == 0xFFFF;
-    strict_w += __popc(__ballot_sync(0xffffffffu, in && (pr || k > kth)));
-    eq_w += __popc(__ballot_sync(0xffffffffu, in && !pr && k == kth));
+  // ---- counts per warp: kept for sure (protected or strictly above the threshold) and ties
+  int strict_w = 0, eq_w = 0;
+#pragma unroll 1
+  for (int i = s0 + lane; i < s1; i += 32) {
+    const bool pr = sSid[i] == 0xFFFF;
+    strict_w += pr || sKey[i] > kth;
+    eq_w += !pr && sKey[i] == kth;
   }
-  // [NW] each, in the second radix pass's histogram buffer (hist + 2048): peers may still be reading the
-  // last pass's buffer (hist[0..]) through DSMEM until barrier (B), but every CTA is done with this one
-  int* seg_strict = hist + 2048;
-  int* seg_eq = hist + 2048 + NW;
+  strict_w = __reduce_add_sync(full, strict_w);
+  eq_w = __reduce_add_sync(full, eq_w);
   if (lane == 0) {
-    seg_strict[warp] = strict_w;
-    seg_eq[warp] = eq_w;
+    w_strict[warp] = strict_w;
+    w_eq[warp] = eq_w;
   }
   __syncthreads();
-  int strict_before = 0, eq_before = 0, strict_cta = 0, eq_cta = 0;  // exclusive prefixes over warps
-  for (int w = 0; w < NW; ++w) {
-    const int sw = seg_strict[w], ew = seg_eq[w];
-    if (w < warp) {
-      strict_before += sw;
-      eq_before += ew;
-    }
-    strict_cta += sw;
-    eq_cta += ew;
-  }
-  if (tid == 0) {
-    ex->loc_keep_base = strict_cta;
-    ex->loc_eq = eq_cta;
-  }
-  cl.sync();  // (B)
-  if (tid < NC) {
-    const int4* rex = reinterpret_cast<const int4*>(cl.peer(ex, tid));
-    const int4 v0 = rex[0], v1 = rex[1];
-    reinterpret_cast<int4*>(&all[tid])[0] = v0;
-    reinterpret_cast<int4*>(&all[tid])[1] = v1;
-  }
-  __syncthreads();
-  // offsets: CTA r keeps its protected + strictly-greater tokens and the ties that fall within the
-  // first need_eq ties in slot order
-  int out_off = 0, total_kept = 0, ties_before = 0, eq_cum = 0, granted_cta = 0;
-  for (int r = 0; r < NC; ++r) {
-    const int granted = max(0, min(need_eq - eq_cum, all[r].loc_eq));
-    const int kept_r = all[r].loc_keep_base + granted;
-    if (r < rank) {
-      out_off += kept_r;
-      ties_before += all[r].loc_eq;
-    }
-    if (r == rank) granted_cta = granted;
-    total_kept += kept_r;
-    eq_cum += all[r].loc_eq;
-  }
-  const bool overflow = total_kept > a.out.kept_cap;
+  const int seg_s = lane < NW ? w_strict[lane] : 0, seg_e = lane < NW ? w_eq[lane] : 0;
+  const int strict_before = __reduce_add_sync(full, lane < warp ? seg_s : 0);
+  const int eq_before = __reduce_add_sync(full, lane < warp ? seg_e : 0);
+  const int eq_cta = __reduce_add_sync(full, seg_e);
+  // a CTA keeps its protected and strictly greater tokens and the ties that fall within the first need_eq in slot order
+  const int prot_pre = min(base, T) - n_pre;
+  const int out_off = prot_pre + strict_pre + min(need_eq, eq_pre);
+  const int granted_cta = max(0, min(need_eq - eq_pre, eq_cta));
   if (rank == 0 && tid == 0) {
     *a.out.n_kept = total_kept;
     if (a.out.n_budget) { a.out.n_budget[0] = N; a.out.n_budget[1] = B; }
     if (overflow) record_status(a.status, STEPKV_ENOSPACE);
   }
 
-  // ---- ordered write of the retained slots: a warp walks its segment in slot order with running
-  // counts (ballot + popc), starting from its segment's prefix within the CTA and the cluster.
+  // ---- ordered write of the retained slots
   if (!overflow) {
-    int tie_rank = ties_before + eq_before;                                 // cluster-wide tie rank
-    int out_pos = out_off + strict_before + min(granted_cta, eq_before);   // next output slot
-    int run_sid = -1, run_c = 0;
+    int tie_rank = eq_pre + eq_before;                                    // cluster-wide tie rank
+    int out_pos = out_off + strict_before + min(granted_cta, eq_before);  // next output slot
     int holes = 0;  // in-place plan: holes among this lane's slots
+    int run_sid = -1, run_c = 0;
+#pragma unroll 1
     for (int i0 = s0; i0 < s1; i0 += 32) {
-      const int i = i0 + lane;
+      const int i = i0 + lane, gi = base + i;
       const bool in = i < s1;
-      const uint32_t k = in ? sKey[i] : 0u;
       const int sid = in ? sSid[i] : 0xFFFF;
-      const bool pr = in && sid == 0xFFFF;
-      const bool is_eq = in && !pr && k == kth;
-      const unsigned lt = (1u << lane) - 1u;
-      const unsigned em = __ballot_sync(0xffffffffu, is_eq);
-      const bool keep = in && (pr || k > kth || (is_eq && tie_rank + __popc(em & lt) < need_eq));
-      const unsigned km = __ballot_sync(0xffffffffu, keep);
+      const uint32_t key = in ? sKey[i] : 0u;
+      const bool pr = in && sid == 0xFFFF, is_eq = in && !pr && key == kth;
+      const unsigned em = __ballot_sync(full, is_eq);
+      const bool keep = pr || (in && (key > kth || (is_eq && tie_rank + __popc(em & lt) < need_eq)));
+      const unsigned km = __ballot_sync(full, keep);
       const int kept_before = out_pos + __popc(km & lt);  // retained slots below this one, cluster-wide
-      if (keep) a.out.kept_idx[kept_before] = base + i;
-      if (a.plan && in && base + i < total_kept) {
-        const int gi = base + i;
-        if (keep) {  // retained in place
-          if (a.step_id_out) a.step_id_out[gi] = __ldg(&a.step_id[gi]);
-          if (a.pos_out) a.pos_out[gi] = a.pos_in ? __ldg(&a.pos_in[gi]) : gi;
-        } else {     // hole number gi - kept_before, filled by the mover of that number
-          a.plan[1 + gi - kept_before] = gi;
-          ++holes;
-        }
+      if (keep) a.out.kept_idx[kept_before] = gi;
+      if (a.plan && in && !keep && gi < total_kept) {  // hole number gi - kept_before, filled by the mover of that number
+        a.plan[1 + gi - kept_before] = gi;
+        ++holes;
       }
       out_pos += __popc(km);
       tie_rank += __popc(em);
@@ -661,25 +644,24 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
         ++run_c;
       }
     }
-    step_stat_flush(run_c > 0, run_sid, run_c, 0ull, 0u, a.acc_kept, nullptr, nullptr);
+    if (want_kept) step_stat_flush(run_c > 0, run_sid, run_c, 0ull, 0u, a.acc_kept, nullptr, nullptr);
     if (a.plan) {
-      for (int o = 16; o > 0; o >>= 1) holes += __shfl_xor_sync(0xffffffffu, holes, o);
+      holes = __reduce_add_sync(full, holes);
       if (lane == 0 && holes) atomicAdd(&a.plan[0], holes);
     }
   }
+  if (NC > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
   if (want_stats || want_kept) {
-    cl.sync();  // (C) all step accumulators final
-
-    // ---- per-step outputs
-    const double fx_unit = ldexp(1.0, -fx_shift);
+    cl.sync();  // all step accumulators final
+    const float fx_unit = __int_as_float((127 - fx_shift) << 23);  // 2^-fx_shift, -85 < fx_shift <= 126
+#pragma unroll 1
     for (int k = rank * NT + tid; k < n_steps; k += NC * NT) {
-      if (a.out.step_count) a.out.step_count[k] = a.acc_cnt[k];
-      if (a.out.step_sal_sum) a.out.step_sal_sum[k] = (float)((double)a.acc_sum[k] * fx_unit);
-      if (a.out.step_sal_max) a.out.step_sal_max[k] = __uint_as_float(a.acc_max[k]);
-      if (a.out.step_kept) a.out.step_kept[k] = a.acc_kept[k];
+      if (a.out.step_count) a.out.step_count[k] = __ldcg(&a.acc_cnt[k]);
+      if (a.out.step_sal_sum) a.out.step_sal_sum[k] = __ull2float_rn(__ldcg(&a.acc_sum[k])) * fx_unit;
+      if (a.out.step_sal_max) a.out.step_sal_max[k] = __uint_as_float(__ldcg(&a.acc_max[k]));
+      if (a.out.step_kept) a.out.step_kept[k] = __ldcg(&a.acc_kept[k]);
     }
   }
-  if (NC > 1) cl.sync();  // no CTA exits while another may still read its shared memory
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -832,13 +814,12 @@ static SelectArgs make_select_args(const SelectSpec& sp) {
   return a;
 }
 
-// Shared memory of one trajectory's CTA: keys + step ids of its chunk, histograms, exchange blocks,
-// scratch, and S_k when it fits.
-static size_t select_smem(int chunk, int nc, int n_steps, int* s_in_smem) {
-  const size_t fixed = (((size_t)chunk * 6 + 15) & ~size_t(15)) + 2 * 2048 * 4 + (1 + nc) * sizeof(SelShared) +
-                       (64 + 2 * (size_t)nc * 64) * 4;
-  const size_t budget_smem = 232448 - 1024;
-  *s_in_smem = fixed + (size_t)n_steps * 4 <= budget_smem ? 1 : 0;
+// Shared memory of one trajectory's CTA: histograms, coarse counts, keys + step ids of its chunk, and S_k when it fits.
+constexpr size_t kSelSmemMax = 232448 - 2048;
+static size_t select_smem(int chunk, int nc, int bits, int n_steps, int* s_in_smem) {
+  const size_t bins = (size_t)1 << bits;
+  const size_t fixed = (2 * bins + 2 * nc * (bins / 32)) * 4 + (size_t)chunk * 6;
+  *s_in_smem = fixed + (size_t)n_steps * 4 <= kSelSmemMax ? 1 : 0;
   return fixed + (*s_in_smem ? (size_t)n_steps * 4 : 0);
 }
 
@@ -848,26 +829,24 @@ stepkv_status_t select_run_batch(const SelectSpec* specs, int n, cudaStream_t st
     int T_max = 0;
     for (int i = 0; i < nb; ++i) T_max = std::max(T_max, specs[b0 + i].T);
     const int nc = T_max <= kSelSingleMaxT ? 1 : kSelClusterCtas;
+    int unused;
+    const int bits = select_smem(((T_max + nc - 1) / nc + 15) & ~15, nc, 13, 0, &unused) <= kSelSmemMax ? 13 : 11;
     SelectBatch batch;
     memset(&batch, 0, sizeof(batch));
     size_t smem = 0;
     for (int i = 0; i < nb; ++i) {
       SelectArgs a = make_select_args(specs[b0 + i]);
       a.chunk = ((a.T + nc - 1) / nc + 15) & ~15;
-      smem = std::max(smem, select_smem(a.chunk, nc, a.steps.n_steps, &a.s_in_smem));
+      smem = std::max(smem, select_smem(a.chunk, nc, bits, a.steps.n_steps, &a.s_in_smem));
       batch.t[i] = a;
     }
-    cudaError_t e;
-    if (nc == 1) {
-      void (*kern)(SelectBatch) = select_kernel<1, 1024>;
-      e = ensure_smem_attr(reinterpret_cast<const void*>(kern), (int)smem);
-      if (e == cudaSuccess) e = launch_kernel(kern, dim3(nb), dim3(1024), smem, stream, batch, true);
-    } else {
-      void (*kern)(SelectBatch) = select_kernel<kSelClusterCtas, 512>;
-      e = ensure_smem_attr(reinterpret_cast<const void*>(kern), (int)smem);
-      if (e == cudaSuccess)
-        e = launch_cluster(kern, dim3(kSelClusterCtas * nb), dim3(512), kSelClusterCtas, smem, stream, batch, true);
-    }
+    void (*kern)(SelectBatch) = nc == 1      ? select_kernel<1, 1024, 13>
+                                : bits == 13 ? select_kernel<kSelClusterCtas, kSelThreads, 13>
+                                             : select_kernel<kSelClusterCtas, kSelThreads, 11>;
+    cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), (int)smem);
+    if (e == cudaSuccess)
+      e = nc == 1 ? launch_kernel(kern, dim3(nb), dim3(1024), smem, stream, batch, true)
+                  : launch_cluster(kern, dim3(nc * nb), dim3(kSelThreads), nc, smem, stream, batch, true);
     if (e != cudaSuccess) {
       set_last_cuda_error(e);
       return STEPKV_ECUDA;

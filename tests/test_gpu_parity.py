@@ -349,6 +349,31 @@ def test_select_exact_on_shared_fp32_priorities(B, levels):
     assert np.array_equal(g.out.step_kept.cpu().numpy(), out["step_kept"])
 
 
+@pytest.mark.parametrize("T", [700, 2048, 2049, 8193, 40000])
+@pytest.mark.parametrize("kind", ["decades", "near_one", "equal", "negated"])
+def test_select_digits(B, kind, T):
+    """The first digit is a linear bin of the priority, the others are digits of the key within that bin: priorities
+    over 30 decades (the threshold in the bin next to zero, whose keys span most of the exponents), a few
+    neighbouring floats near one, one value only, and a descending order (alpha < 0).  The kernel ranks exactly the fp32
+    values it is given, so the retained set equals the oracle's bit for bit at every budget."""
+    import torch
+    tr = wl.custom(9, L=1, Hq=1, Hkv=1, d=64, T=T, W=8, n_steps=5)
+    rng = np.random.default_rng(T)
+    sal = {"decades": np.exp(rng.uniform(-69.0, 0.0, T)), "near_one": 1.0 + rng.integers(0, 5, T) * 2.0**-23,
+           "equal": np.full(T, 0.37), "negated": rng.random(T)}[kind].astype(np.float32)
+    alpha = -1.0 if kind == "negated" else 1.0
+    p = B.Params(alpha=alpha, beta=0.0, sal_norm=B.NORM_NONE)
+    prunable = ~tr.prot.astype(bool)
+    for count in (1, T // 3, T - 200):
+        tr.budget = wl.Budget.fixed(count)
+        g, out, st = _select_case(B, tr, p, sal[None])
+        assert st == 0
+        gk = g.out.kept_idx[:int(g.out.n_kept.item())].cpu().numpy()
+        want = O.kept_indices(tr.prot, O.select_top(alpha * sal.astype(np.float64), prunable,
+                                                    O.budget_tokens(int(prunable.sum()), "count", count=count)))
+        assert np.array_equal(gk, want), (kind, T, count)
+
+
 @pytest.mark.parametrize("pool, mode, T", [(3, 0, 9000), (7, 0, 9000), (7, 1, 9000), (63, 1, 9000), (31, 0, 9000),
                                            (5, 1, 1500)])
 def test_select_snapkv_pooling(B, pool, mode, T):
