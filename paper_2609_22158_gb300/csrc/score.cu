@@ -167,8 +167,8 @@ struct ScoreCfg {
   static constexpr int kTabOff = kQBytes + kStages * kStageBytes;     // float negoff[2][256] | int pw[2][256]
   static constexpr int kCombOff = kTabOff + 2 * 2 * kMaxRows * 4;    // | float comb[2 grp][2 parity][128]
   static constexpr int kBarOff = kCombOff + 2 * 2 * 128 * 4;
-  // k_full/k_empty per stage, q_full/q_empty, acc_full/acc_empty[2], epi[2], p1_flushed
-  static constexpr int kNumBars = 2 * kStages + 2 + 4 + 2 + 1;
+  // k_full/k_empty per stage, q_full/q_empty, acc_full/acc_empty[2], epi[2], p1_flushed, comb_full[8]
+  static constexpr int kNumBars = 2 * kStages + 2 + 4 + 2 + 1 + 8;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;                 // tmem base, abort flag
   static constexpr int kBytes = kMiscOff + 16;
   static constexpr int kDynSmem = kBytes + 1024;                          // + alignment slack
@@ -269,25 +269,26 @@ __device__ __forceinline__ void row_stats_update(const float (&va)[32], const fl
 // 0-15, rb: lanes 16-31).  Register 4k + e of a load holds lane lane/4 + 8 (e >= 2) and column
 // 8k + 2 (lane % 4) + (e & 1), so a thread sees 4 keys, lane/4 + 8 kk (kk < 4), and 8 columns of the
 // chunk, whose offsets o2[k] (pairs of columns) it loaded from the unit's table.  acc2[kk] collects
-// 2^(s c - off_r) over those columns for key kk in pairs; columns whose causal limit pw_r is below the
-// key contribute nothing (only tiles that reach into the window need the test, jq = key of kk = 0).
+// 2^(s c - off_r) over those columns for key kk in pairs; in the masked form, columns whose causal limit pw_r is
+// below the key contribute nothing (jq = key of kk = 0).
 __device__ __forceinline__ void chunk_mass(const uint32_t (&ra)[16], const uint32_t (&rb)[16], const uint64_t (&o2)[4],
-                                           const int* pw, int jq, bool need_mask, float c, uint64_t (&acc2)[4]) {
-  if (!need_mask) {
-    const uint64_t c2 = f2_pack(c, c);
+                                           float c, uint64_t (&acc2)[4]) {
+  const uint64_t c2 = f2_pack(c, c);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < 4; ++k) {
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t* r = kk < 2 ? ra : rb;
-        const int e = 4 * k + (kk & 1) * 2;
-        float lo, hi;
-        f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), c2, o2[k]), lo, hi);
-        acc2[kk] = f2_add(acc2[kk], f2_pack(ex2_approx(lo), ex2_approx(hi)));
-      }
+    for (int kk = 0; kk < 4; ++kk) {
+      const uint32_t* r = kk < 2 ? ra : rb;
+      const int e = 4 * k + (kk & 1) * 2;
+      float lo, hi;
+      f2_unpack(f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), c2, o2[k]), lo, hi);
+      acc2[kk] = f2_add(acc2[kk], f2_pack(ex2_approx(lo), ex2_approx(hi)));
     }
-    return;
   }
+}
+__device__ __forceinline__ void chunk_mass_masked(const uint32_t (&ra)[16], const uint32_t (&rb)[16],
+                                                  const uint64_t (&o2)[4], const int* pw, int jq, float c,
+                                                  uint64_t (&acc2)[4]) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int2 w = *reinterpret_cast<const int2*>(&pw[8 * k]);
@@ -345,7 +346,6 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
   uint8_t* sQ = sm;
   uint8_t* sK = sm + Cfg::kQBytes;
   float* sNegOff = reinterpret_cast<float*>(sm + Cfg::kTabOff);
-  int* sPw = reinterpret_cast<int*>(sm + Cfg::kTabOff + 2 * kMaxRows * 4);
   float* sComb = reinterpret_cast<float*>(sm + Cfg::kCombOff);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + Cfg::kBarOff);
   uint64_t* k_full = bars;
@@ -356,6 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
   uint64_t* acc_empty = acc_full + 2;  // [2]
   uint64_t* epi_bar = acc_empty + 2;   // [2], one per epilogue group
   uint64_t* p1_flushed = epi_bar + 2;  // every epilogue warp has written its pass-1 partials
+  uint64_t* comb_full = p1_flushed + 1;  // [2 grp][4 quarters]: the second warp's share of an item (rows output)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + Cfg::kMiscOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + Cfg::kMiscOff + 4);
 
@@ -383,6 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
       mbar_init(&epi_bar[b], kGroupWarps);
     }
     mbar_init(p1_flushed, kEpiWarps);
+    for (int i = 0; i < 8; ++i) mbar_init(&comb_full[i], 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -600,7 +602,6 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
     // The per-token accumulators (8 bytes per token) take an atomic per key and KV head in pass 2; an
     // evict-last L2 policy on their zeroing stores and atomics keeps them resident while the key tiles
     // stream through L2 (fused pass 279.6 -> 277.7 us at T = 32768).
-    const uint64_t acc_pol = l2_policy_evict_last();
     // The first epilogue warp zeroes this CTA's share of the accumulators (when the launch accumulates)
     // while the first tiles stream in, then publishes its zero flag (fence + release store of the launch
     // token): a CTA adds into the accumulators only after it has seen every CTA's zero flag, and CTA 0
@@ -609,7 +610,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
       if (p.accumulate) {
         for (int b = 0; b < p.n_traj; ++b) {
           unsigned long long* acc = p.traj[b].t_acc;
-          for (int i = blockIdx.x * 32 + lane; i < p.traj[b].T; i += gridDim.x * 32) st_u64_hint(acc + i, 0ull, acc_pol);
+          for (int i = blockIdx.x * 32 + lane; i < p.traj[b].T; i += gridDim.x * 32) st_u64_hint(acc + i, 0ull, l2_policy_evict_last());
         }
       }
       __syncwarp();
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
     // ---- pass 1: per-row running (m, Z) over the keys this warp sees (skipped when the caller gives the
     // rows' log-sum-exp)
     if (!p.pass2_only) {
-      int cur = -1, Tb = 0;
+      int cur = -1, lim = 0;  // lim: the last key that every row of the warp sees
       float m = -INFINITY, Z = 0.f;
       int my_row = 0, my_pw = 0, my_e = 0;
       bool row_ok = false, two = false;
@@ -636,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
         const int u = il.u, tile = il.tile;
         t += nt;
         if (u != cur) {
-          Tb = p.traj[il.b].T;
+          const int Tb = p.traj[il.b].T;
           // Every warp flushes every unit the CTA touches (an untouched share flushes m = -inf, Z = 0),
           // so each of the unit's partial entries is written.
           if (cur >= 0) flush_partial(cur);
@@ -651,6 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
           const int w = r.w0 + my_row % r.blk_rows;
           row_ok = my_row < r.rows && w < g.W;
           my_pw = Tb - g.W + w;
+          lim = Tb - g.W + (g.split ? r.w0 + mt_g * 128 + q * 32 : 0);  // a split head's rows are consecutive
           m = -INFINITY;
           Z = 0.f;
           cur = u;
@@ -666,7 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
         // chunks (one TMEM round trip per pair); the buffer is released once the last pair is loaded.
         const int half_keys = nt * 64;
         const int key0 = tile * kKeyTile + s2 * half_keys;
-        const bool need_mask = key0 + half_keys - 1 > Tb - g.W;  // reaches into the causal window
+        const bool need_mask = key0 + half_keys - 1 > lim;
         const int n_pairs_ch = half_keys / 64;
 #pragma unroll 1
         for (int h2 = 0; h2 < n_pairs_ch; ++h2) {
@@ -677,6 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
           if (row_ok) {
             const int j0 = key0 + h2 * 64;
             if (need_mask) {
+              if (j0 > my_pw) continue;  // this row sees none of the chunk's keys
 #pragma unroll
               for (int i = 0; i < 32; ++i) {
                 va[i] = (j0 + i <= my_pw) ? va[i] : -INFINITY;
@@ -709,10 +712,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
     // ---- pass 2: per-key mass over the query rows, with the offsets of every row of the unit
     if (ok) {
       int cur = -1, n_done = 0;  // n_done: pass-2 items this group has drained
-      RowGroup r{};
+      int n_cols = 0, lim = 0;  // lim: the last key that every row of the unit sees
       bool zeros_seen = !p.accumulate;
       float* negoff = sNegOff + grp * kMaxRows;  // this group's per-row offsets and causal limits
-      int* pw_tab = sPw + grp * kMaxRows;
       float* combf = sComb + grp * (2 * 128);     // rows output: [2 parity][128]
       // pass-2 item k is half hh + k: this group drains every other item, starting with the first of its parity
       const int k_first = (int)(((uint32_t)grp - hh) & 1u);
@@ -753,7 +755,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
           // Combine the pass-1 partials of unit u into this group's per-row offsets, in contributing-CTA
           // order (the group no longer reads the previous unit's offsets once all its warps arrive).
           if (!(ok = epi_sync(&epi_bar[grp], eb_phase, abort_flag))) break;
-          r = row_group(g, fmodulo(u, g.rg_div));
+          const RowGroup r = row_group(g, fmodulo(u, g.rg_div));
+          n_cols = (r.rows + 31) & ~31;
+          lim = Tb - g.W + r.w0;  // (w0 > 0: a split head's rows are consecutive window offsets)
           const int n_e = r.rows > 128 ? 2 : kPartEntries;  // entries written per row in pass 1
           const int n_e_log2 = r.rows > 128 ? 1 : 2;
           const int row = (ew & 7) * 32 + lane;             // 256 threads of the group, one row each
@@ -796,7 +800,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
             off = M * c + __log2f(Zs);
           }
           negoff[row] = -off;
-          pw_tab[row] = valid ? Tb - g.W + w : -1;
+          reinterpret_cast<int*>(negoff + 2 * kMaxRows)[row] = valid ? Tb - g.W + w : -1;
           if (!(ok = epi_sync(&epi_bar[grp], eb_phase, abort_flag))) break;
           cur = u;
         }
@@ -804,27 +808,48 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
         acc_phase ^= 1;
         tc_fence_after();
         const int key0 = tile * kKeyTile;
-        const bool need_mask = key0 + kKeyTile - 1 > Tb - g.W;  // tile reaches into the causal window
+        const bool need_mask = key0 + kKeyTile - 1 > lim;  // some row does not see some key of the tile
         // Keys on the TMEM lanes: this warp covers its quarter's 32 keys over query columns s2*32 + 64 i
         // (32-column chunks, one TMEM round trip each; holding two chunks in registers spills).  Per
         // chunk a thread needs 8 row offsets, so the shared-memory reads per logit drop fourfold against
         // the one-key-per-thread 32x32b layout.  The buffer is released once the warp's last chunk is in
         // registers.
-        const int n_cols = (r.rows + 31) & ~31;
         const int lq = lane & 3;
-        const int jq = key0 + q * 32 + (lane >> 2);
         uint64_t acc2[4] = {0ull, 0ull, 0ull, 0ull};
+        auto load_chunk = [&](int cc, uint64_t (&o2)[4], uint32_t (&ra)[16], uint32_t (&rb)[16]) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int cc = s2 * 32 + 64 * i;
-          if (cc < n_cols) {
+          for (int k = 0; k < 4; ++k) o2[k] = *reinterpret_cast<const uint64_t*>(&negoff[cc + 8 * k + 2 * lq]);
+          tmem_ld16x256x4_pair(lane_base + (uint32_t)cc, lane_base + (16u << 16) + (uint32_t)cc, ra, rb);
+          if (cc + 64 >= n_cols) release_buffer();
+        };
+        // The masked chunks have a rolled loop of their own and find their limits from the offsets' address: beside the
+        // unmasked ones in one unrolled loop they cost every tile registers and code (fused pass at T = 32768 258.0 ->
+        // 255.0 us; without any masked path 252.5).  Only tiles past `lim` take it, and a chunk none of whose columns
+        // sees the warp's keys is skipped: a 2048-row window's saliency 2687 -> 2594 us.
+        if (!need_mask) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int cc = s2 * 32 + 64 * i;
+            if (cc < n_cols) {
+              uint64_t o2[4];
+              uint32_t ra[16], rb[16];
+              load_chunk(cc, o2, ra, rb);
+              chunk_mass(ra, rb, o2, c, acc2);
+            }
+          }
+        } else {
+          const int* pw = reinterpret_cast<const int*>(negoff + 2 * kMaxRows);
+          const int j_lo = key0 + q * 32;  // the warp's first key
+#pragma unroll 1
+          for (int cc = s2 * 32; cc < n_cols; cc += 64) {
+            if (__all_sync(0xffffffffu, pw[cc + lane] < j_lo)) {  // no column of the chunk sees any of the keys
+              if (cc + 64 >= n_cols) release_buffer();
+              continue;
+            }
             uint64_t o2[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) o2[k] = *reinterpret_cast<const uint64_t*>(&negoff[cc + 8 * k + 2 * lq]);
             uint32_t ra[16], rb[16];
-            tmem_ld16x256x4_pair(lane_base + (uint32_t)cc, lane_base + (16u << 16) + (uint32_t)cc, ra, rb);
-            if (cc + 64 >= n_cols) release_buffer();
-            chunk_mass(ra, rb, o2, pw_tab + cc + 2 * lq, jq, need_mask, c, acc2);
+            load_chunk(cc, o2, ra, rb);
+            chunk_mass_masked(ra, rb, o2, pw + cc + 2 * lq, j_lo + (lane >> 2), c, acc2);
           }
         }
         if (s2 * 32 >= n_cols) release_buffer();  // no chunk for this warp
@@ -845,13 +870,21 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
         if (p.accumulate) {
           // fused pass: each warp adds its share of the rows straight into the per-token fixed-point
           // sum (integer addition: the total does not depend on the order of arrival)
-          if (j < Tb) red_add_u64_hint(&p.traj[il.b].t_acc[j], to_fixed(acc * g.inv_G, p.acc_shift), acc_pol);
+          if (j < Tb) red_add_u64_hint(&p.traj[il.b].t_acc[j], to_fixed(acc * g.inv_G, p.acc_shift),
+                                       l2_policy_evict_last());
         } else {
-          // saliency rows: the group's two warps on this quarter combine in a fixed order (the slot
-          // alternates between the group's items, so a write never meets a pending read)
+          // saliency rows: the group's two warps on this quarter combine in a fixed order.  The second hands its
+          // share over and goes on; the slot alternates between the group's items, and it cannot reach the item after
+          // next before the first has released that item's accumulator, which it does after this item's read.
           float* comb = combf + (n_done & 1) * 128;
-          if (s2 == 1) comb[q * 32 + lk] = acc;
-          if (!(ok = epi_sync(&epi_bar[grp], eb_phase, abort_flag))) break;
+          uint64_t* bar = comb_full + grp * 4 + q;
+          if (s2 == 1) {
+            comb[q * 32 + lk] = acc;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar);
+          } else if (!(ok = mbar_wait(bar, (uint32_t)n_done & 1u, abort_flag))) {
+            break;
+          }
           if (s2 == 0 && j < Tb) {
             const float val = (acc + comb[q * 32 + lk]) * g.inv_G;
             int rg;

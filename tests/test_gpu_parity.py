@@ -60,6 +60,23 @@ def test_score_matches_oracle(B, Hkv, G, d, T, W, nl):
         assert np.allclose(g[l].sum(axis=1), W, rtol=1e-4)
 
 
+@pytest.mark.parametrize("Hkv,G,d,T,W", [(1, 2, 64, 1300, 777), (1, 1, 128, 1024, 1024), (2, 3, 64, 901, 600),
+                                         (1, 1, 128, 385, 257)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_score_split_window_masks(B, Hkv, G, d, T, W, lse):
+    """Windows split over row groups at odd lengths: tiles that every row of a group sees, that straddle its causal limits,
+    and that no row (or no row of a warp or of a chunk) sees, in both passes."""
+    import torch
+    rng = np.random.default_rng(T * 7 + W)
+    k, q = _rand_bits(rng, (Hkv, T, d), 2.0), _rand_bits(rng, (Hkv * G, W, d))
+    stats = [torch.from_numpy(O.window_row_lse(k, q).astype(np.float32)).cuda()] if lse else None
+    st = B.new_status()
+    sal = B.stepkv_score([TL.bf16_dev(k)], [TL.bf16_dev(q)], T, status=st, lse=stats)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    TL.assert_close(sal[0].cpu().numpy(), O.window_attention_saliency(k, q), "sal")
+
+
 @pytest.mark.parametrize("Hkv,G,d,T,W,nl", SCORE_CASES + [(1, 4, 128, 2500, 512, 1), (1, 5, 128, 3000, 1024, 1)])
 def test_score_with_prefill_lse_matches_oracle(B, Hkv, G, d, T, W, nl):
     """stepkv_score_lse: the rows' log-sum-exp comes from the caller (the oracle's, rounded to fp32, as
