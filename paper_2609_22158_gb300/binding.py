@@ -204,7 +204,11 @@ def _rows_layout(ts: Sequence, name: str, host=False):
     """[H, rows, d] bf16 tensors with unit stride in d and dense rows; returns (head_stride, rows)."""
     torch = _torch()
     hs = None
+    same = None  # the previous tensor's layout, checked: a tensor laid out the same needs no checks of its own
     for i, t in enumerate(ts):
+        lay = None if host else _layout(torch, t)
+        if lay is not None and lay == same:
+            continue
         _need(t, torch.bfloat16, f"{name}[{i}]", 3, host=host)
         H, R, d = t.shape
         if t.stride(2) != 1 or (R > 1 and t.stride(1) != d):
@@ -214,14 +218,32 @@ def _rows_layout(ts: Sequence, name: str, host=False):
             hs = s
         elif hs != s:
             raise ValueError(f"all {name} tensors must share one head stride")
+        same = lay
     return hs
 
 
-def _ptr_array(ts) -> ctypes.Array:
-    arr = (ctypes.c_void_p * max(1, len(ts)))()
+def _layout(torch, t):
+    """What the argument checks of a per-layer tensor look at, in five attribute reads: two tensors for which it is equal
+    pass or fail them alike.  None for anything but a CUDA tensor.  (A decode call of 64 layers checks 320 tensors;
+    check by check that took longer than the read itself takes on the GPU.)"""
+    if isinstance(t, torch.Tensor) and t.is_cuda:
+        return t.dtype, t.shape, t.stride()
+    return None
+
+
+def _need_all(ts, check, name):
+    """check(t, name) for every per-layer tensor laid out differently from the one checked before it."""
+    torch = _torch()
+    same = None
     for i, t in enumerate(ts):
-        arr[i] = t.data_ptr()
-    return arr
+        lay = _layout(torch, t)
+        if lay is None or lay != same:
+            check(t, f"{name}[{i}]")
+            same = lay
+
+
+def _ptr_array(ts) -> ctypes.Array:
+    return (ctypes.c_void_p * max(1, len(ts)))(*[t.data_ptr() for t in ts])
 
 
 def new_status(device=None):
@@ -411,6 +433,16 @@ def stepkv_select(sal, step_id, prot, steps: StepSignals, params: Params, budget
 
 
 # ----------------------------------------------------------------------------- decode attention
+def _check_q(t, name):
+    _need(t, _torch().bfloat16, name, 2)
+    if not t.is_contiguous():
+        raise ValueError(f"{name} must be contiguous")
+
+
+def _check_f32_2d(t, name):
+    _need(t, _torch().float32, name, 2)
+
+
 def stepkv_decode(q: Sequence, K: Sequence, V: Sequence, n, out: Optional[Sequence] = None, ws=None, status=None,
                   stream=None):
     """One query token per layer over a (compacted) cache: out[l][g] = softmax(q[l][g] K^T / sqrt(d)) V.
@@ -424,16 +456,12 @@ def stepkv_decode(q: Sequence, K: Sequence, V: Sequence, n, out: Optional[Sequen
         raise ValueError("q, K and V need one tensor per layer")
     hs = _rows_layout(list(K) + list(V), "K/V")
     Hkv, rows, d = K[0].shape
-    for i, t in enumerate(q):
-        _need(t, torch.bfloat16, f"q[{i}]", 2)
-        if not t.is_contiguous():
-            raise ValueError(f"q[{i}] must be contiguous")
+    _need_all(q, _check_q, "q")
     Hq = q[0].shape[0]
     dev = q[0].device
     if out is None:
         out = [torch.empty((Hq, d), dtype=torch.float32, device=dev) for _ in range(L)]
-    for i, t in enumerate(out):
-        _need(t, torch.float32, f"out[{i}]", 2)
+    _need_all(out, _check_f32_2d, "out")
     if isinstance(n, int):
         n_dev, n_host = None, n
     else:
@@ -462,20 +490,19 @@ def stepkv_decode_h2o(q: Sequence, K: Sequence, V: Sequence, n, mass: Sequence, 
         raise ValueError("q, K, V and mass need one tensor per layer")
     hs = _rows_layout(list(K) + list(V), "K/V")
     Hkv, rows, d = K[0].shape
-    for i, t in enumerate(q):
-        _need(t, torch.bfloat16, f"q[{i}]", 2)
-        if not t.is_contiguous():
-            raise ValueError(f"q[{i}] must be contiguous")
-    for i, t in enumerate(mass):
-        _need(t, torch.float32, f"mass[{i}]", 2)
+    _need_all(q, _check_q, "q")
+
+    def check_mass(t, name):
+        _check_f32_2d(t, name)
         if t.shape[0] != Hkv or t.shape[1] < rows or t.stride(1) != 1 or t.stride(0) != mass[0].stride(0):
             raise ValueError("mass[l] must be [Hkv, >= rows] float32 with unit column stride and one row stride")
+
+    _need_all(mass, check_mass, "mass")
     Hq = q[0].shape[0]
     dev = q[0].device
     if out is None:
         out = [torch.empty((Hq, d), dtype=torch.float32, device=dev) for _ in range(L)]
-    for i, t in enumerate(out):
-        _need(t, torch.float32, f"out[{i}]", 2)
+    _need_all(out, _check_f32_2d, "out")
     if isinstance(n, int):
         n_dev, n_host = None, n
     else:

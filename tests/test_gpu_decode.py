@@ -130,3 +130,28 @@ def test_decode_stream_split(B, G, d, h2o, n):
         assert torch.equal(same, out)
         TL.assert_close(mass[0][:, :n].cpu().numpy(), O.decode_attention_mass(q, K), "mass", floor=1e-30)
         assert not mass[0][:, n:].any()
+
+
+def test_decode_rejects_one_bad_layer_among_many(B):
+    """Layers laid out alike are checked once: one that differs, wherever it stands, is still found."""
+    import torch
+    L, Hkv, G, d, rows = 4, 2, 4, 64, 96
+    z = lambda *s, **k: torch.zeros(s, device="cuda", **k)
+    bf = torch.bfloat16
+    good = dict(q=lambda: [z(Hkv * G, d, dtype=bf) for _ in range(L)], K=lambda: [z(Hkv, rows, d, dtype=bf) for _ in range(L)],
+                V=lambda: [z(Hkv, rows, d, dtype=bf) for _ in range(L)], mass=lambda: [z(Hkv, rows) for _ in range(L)],
+                out=lambda: [z(Hkv * G, d) for _ in range(L)])
+    bad = [("q", z(d, Hkv * G, dtype=bf).T, ValueError), ("q", z(Hkv * G, d), TypeError), ("q", z(Hkv * G, d, dtype=bf).cpu(), ValueError),
+           ("K", z(Hkv, 2 * rows, d, dtype=bf)[:, :rows], ValueError), ("V", z(Hkv, rows, 2 * d, dtype=bf)[:, :, ::2], ValueError),
+           ("K", z(Hkv, rows, d), TypeError), ("V", z(Hkv, rows, d, dtype=bf).cpu(), ValueError),
+           ("mass", z(Hkv, rows, dtype=torch.float64), TypeError), ("mass", z(Hkv, rows - 1), ValueError),
+           ("mass", z(Hkv, 2 * rows)[:, :rows], ValueError), ("out", z(Hkv * G, d, dtype=bf), TypeError), ("out", z(Hkv * G * d), ValueError)]
+    for name, tensor, err in bad:
+        for at in (1, L - 1):
+            a = {k: f() for k, f in good.items()}
+            a[name][at] = tensor
+            with pytest.raises(err):
+                B.stepkv_decode_h2o(a["q"], a["K"], a["V"], rows, a["mass"], out=a["out"])
+    a = {k: f() for k, f in good.items()}
+    B.stepkv_decode_h2o(a["q"], a["K"], a["V"], rows, a["mass"], out=a["out"])
+    torch.cuda.synchronize()
