@@ -718,6 +718,37 @@ def test_compress_in_place_hole_filling(B, T, num, den, all_prot):
         assert np.array_equal(TL.bits_of(g.V[l])[:, :n], src[1][l][:, exp])
 
 
+def test_compress_in_place_many_moves(B):
+    """More row moves per CTA than its shared memory stages at a time (1.5 million moves of 128-byte rows), against a
+    gather of the original rows by the positions the call reports."""
+    import torch
+    L, Hkv, d, T = 32, 16, 64, 6000
+    tr = wl.custom(31, L=1, Hq=16, Hkv=16, d=d, T=T, W=16, n_steps=8, budget=wl.Budget.ratio(1, 2))
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda", dtype=torch.bfloat16)
+    KV = rnd(2, L, Hkv, T, d)
+    was = KV.clone()
+    t = lambda a: torch.from_numpy(a).cuda()
+    steps = B.StepSignals(t(tr.valid), t(tr.gain), t(tr.red), t(tr.reuse), t(tr.obs_sim))
+    out = B.SelectOutputs.allocate(T, tr.n_steps, T, "cuda", full=False)
+    pos_out = torch.full((T,), -1, dtype=torch.int32, device="cuda")
+    K, V = list(KV[0]), list(KV[1])
+    prob = B.Problem(K, V, [rnd(16, 16, d) for _ in range(3)], T, t(tr.step_id), t(tr.prot), steps, B.budget_ratio(1, 2),
+                     K, V, out, pos_out=pos_out)
+    st = B.stepkv_compress([prob], B.Params(alpha=1.0, beta=0.0))
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    n = int(out.n_kept.item())
+    kept = out.kept_idx[:n]
+    assert int((kept >= n).sum()) * 2 * L * Hkv > 1024 * 1216  # every CTA stages more than once
+    stay = torch.zeros(n, dtype=torch.bool, device="cuda")
+    stay[kept[kept < n].long()] = True
+    src = torch.arange(n, device="cuda")
+    src[~stay] = kept[kept >= n].long()
+    assert torch.equal(pos_out[:n].long(), src)
+    assert torch.equal(KV[:, :, :, :n], was[:, :, :, src]) and torch.equal(KV[:, :, :, n:], was[:, :, :, n:])
+
+
 def test_compress_in_place_overflow_moves_nothing(B):
     """In place with kept_cap below the retained count (Eq. 1's protected + budget rows): the call records
     STEPKV_ENOSPACE on the device, lays out no plan, and leaves every layer's cache rows and the step /
