@@ -244,6 +244,13 @@ __device__ __forceinline__ unsigned long long to_fixed(float x, int shift) {
   return (mant + (1ull << (-sh - 1))) >> (-sh);
 }
 
+// The smaller of the two, NaN where either is.
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // Float <-> order-preserving unsigned key (larger float <=> larger key; -0 < +0).
 __device__ __forceinline__ uint32_t float_to_ordered(float f) {
   uint32_t u = __float_as_uint(f);

@@ -33,6 +33,7 @@ namespace stepkv {
 constexpr int kSelSingleMaxT = 2048;
 constexpr int kSelClusterCtas = 8;
 constexpr int kSelThreads = 1024;
+constexpr uint32_t kNanKey = 0x007FFFFEu;  // just below the key of -inf
 
 struct SelectArgs {
   const float* T_in;                  // token saliency as floats, or
@@ -65,7 +66,7 @@ struct SelectArgs {
 
 // One CTA's summary, pushed into every CTA of the cluster.
 struct SelSummary {
-  float max_T, min_T;  // over prunable tokens
+  float max_T, min_T;  // over prunable tokens (min_T: NaN where one is)
   int n;               // prunable tokens
   int err;
 };
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
         sT[i] = tv[u];
         if (sSid[i] != 0xFFFFu) {
           lmax = fmaxf(lmax, tv[u]);
-          lmin = fminf(lmin, tv[u]);
+          lmin = min_nan(lmin, tv[u]);
         }
       }
     }
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     lmax = fmaxf(lmax, __shfl_xor_sync(full, lmax, o));
-    lmin = fminf(lmin, __shfl_xor_sync(full, lmin, o));
+    lmin = min_nan(lmin, __shfl_xor_sync(full, lmin, o));
   }
   if (lane == 0) {
     w_max[warp] = lmax;
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       m = fmaxf(m, __shfl_xor_sync(full, m, o));
-      mi = fminf(mi, __shfl_xor_sync(full, mi, o));
+      mi = min_nan(mi, __shfl_xor_sync(full, mi, o));
       b_lo = fminf(b_lo, __shfl_xor_sync(full, b_lo, o));
       b_hi = fmaxf(b_hi, __shfl_xor_sync(full, b_hi, o));
     }
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
 #pragma unroll
   for (int r = 0; r < NC; ++r) {
     gmax = fmaxf(gmax, all[r].max_T);
-    gmin = fminf(gmin, all[r].min_T);
+    gmin = min_nan(gmin, all[r].min_T);
     if (r < rank) n_pre += all[r].n;
     N += all[r].n;
     err |= all[r].err;
@@ -375,8 +376,14 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
 
   // ---- priorities (Eq. 5) and their bounds; bins of the first digit
   const float t_lo = gmin * inv_max, t_hi = gmax * inv_max;
-  const float P_lo = fminf(fmaf(a.prm.alpha, t_lo, s_lo[0]), fmaf(a.prm.alpha, t_hi, s_lo[0]));
-  const float P_hi = fmaxf(fmaf(a.prm.alpha, t_lo, s_hi[0]), fmaf(a.prm.alpha, t_hi, s_hi[0]));
+  float P_lo = fminf(fmaf(a.prm.alpha, t_lo, s_lo[0]), fmaf(a.prm.alpha, t_hi, s_lo[0]));
+  float P_hi = fmaxf(fmaf(a.prm.alpha, t_lo, s_hi[0]), fmaf(a.prm.alpha, t_hi, s_hi[0]));
+  // Where a priority can lie outside them (a saliency that is not finite, an overflow) the bounds become the infinities:
+  // all keys share the first bin and their whole 32 bits follow.  A priority that is not a number ranks below -inf.
+  if (!(fabsf(gmin) < INFINITY && fabsf(gmax) < INFINITY && fabsf(P_lo) < INFINITY && fabsf(P_hi) < INFINITY)) {
+    P_lo = -INFINITY;
+    P_hi = INFINITY;
+  }
   const float scale = P_hi > P_lo ? 0.999999f * (float)kBins / (P_hi - P_lo) : 0.f;
   auto first_bin = [&](uint32_t key) {  // monotone in the priority
     return min(max((int)((ordered_to_float(key) - P_lo) * scale), 0), kBins - 1);
@@ -397,7 +404,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
       float P = -INFINITY;
       if (sid != 0xFFFF) {
         P = fmaf(a.prm.alpha, x, a.prm.beta * Sk[sid]);
-        key = float_to_ordered(P);
+        key = P == P ? float_to_ordered(P) : kNanKey;
         if (want_stats) {
           const float xc = fmaxf(x, 0.f);
           if (sid != run_sid) {
@@ -561,7 +568,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
         // the keys of the bin lie within its bounds, widened by its rounding and two keys
         star = digit;
         uint32_t k_hi = float_to_ordered(P_hi);
-        k_lo = float_to_ordered(P_lo);
+        k_lo = float_to_ordered(P_lo) - 1u;  // below -inf: kNanKey
         const float w = 1.0f / scale;
         if (scale > 0.f && w > 0.f) {
           const uint32_t lo = float_to_ordered(P_lo + ((float)star - 0.02f) * w) - 2u;

@@ -391,6 +391,43 @@ def test_select_digits(B, kind, T):
         assert np.array_equal(gk, want), (kind, T, count)
 
 
+@pytest.mark.parametrize("T", [1000, 9000])
+@pytest.mark.parametrize("kind", ["nan", "inf", "both", "all_nan", "overflow"])
+def test_select_non_finite_saliency(B, kind, T):
+    """Saliency values that are not finite, or priorities that overflow: no bounds hold all priorities then, so the first
+    digit tells nothing and the whole key decides, NaN below -inf.  A budget above the prunable tokens keeps them all."""
+    import torch
+    tr = wl.custom(9, L=1, Hq=1, Hkv=1, d=64, T=T, W=8, n_steps=5)
+    rng = np.random.default_rng(T)
+    sal = rng.random(T).astype(np.float32)
+    pick = rng.permutation(T)
+    if kind in ("nan", "both"):
+        sal[pick[:40]] = np.nan
+    if kind in ("inf", "both"):
+        sal[pick[40:90]], sal[pick[90:150]] = np.inf, -np.inf
+    if kind == "all_nan":
+        sal[:] = np.nan
+    alpha = np.float32(1.0)
+    if kind == "overflow":
+        alpha = np.float32(2.0)
+        sal = np.where(rng.random(T) < 0.3, np.float32(3e38), sal).astype(np.float32)
+    with np.errstate(over="ignore"):
+        prio = alpha * sal
+    bits = prio.view(np.uint32)
+    key = np.where(np.isnan(prio), 1, np.where(bits >> 31, ~bits, bits | np.uint32(0x80000000))).astype(np.int64)
+    prunable = ~tr.prot.astype(bool)
+    p = B.Params(alpha=float(alpha), beta=0.0, sal_norm=B.NORM_NONE)
+    step_id, prot = torch.from_numpy(tr.step_id).cuda(), torch.from_numpy(tr.prot).cuda()
+    steps = B.StepSignals(*(torch.from_numpy(a).cuda() for a in (tr.valid, tr.gain, tr.red, tr.reuse)))
+    for count in (1, 30, T // 3, T - 200, T - 40, T):
+        out, st = B.SelectOutputs.allocate(T, tr.n_steps, T, "cuda"), B.new_status()
+        B.stepkv_select(torch.from_numpy(sal[None]).cuda(), step_id, prot, steps, p, B.budget_count(count), out, status=st)
+        assert int(st.item()) == 0
+        order = sorted(np.flatnonzero(prunable), key=lambda i: (-key[i], i))
+        want = np.sort(np.concatenate([np.flatnonzero(~prunable), order[:count]])).astype(np.int64)
+        assert np.array_equal(out.kept_idx[:int(out.n_kept.item())].cpu().numpy(), want), (kind, T, count)
+
+
 @pytest.mark.parametrize("pool, mode, T", [(3, 0, 9000), (7, 0, 9000), (7, 1, 9000), (63, 1, 9000), (31, 0, 9000),
                                            (5, 1, 1500)])
 def test_select_snapkv_pooling(B, pool, mode, T):
