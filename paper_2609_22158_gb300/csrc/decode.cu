@@ -193,7 +193,7 @@ struct DecodeState {
     mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
     if (__any_sync(0xffffffffu, mb > m)) {
       const float mn = fmaxf(m, mb);
-      const float sc = ex2_approx((m - mn) * c);
+      const float sc = m == mn ? 1.f : ex2_approx((m - mn) * c);  // (both -inf: no key of this head yet)
       const uint64_t sc2 = f2_pack(sc, sc);
       l *= sc;
 #pragma unroll
@@ -202,7 +202,7 @@ struct DecodeState {
         for (int t = 0; t < 8; ++t) acc[s2][t] = f2_mul(acc[s2][t], sc2);
       m = mn;
     }
-    const float mc = m * c;
+    const float mc = m == -INFINITY ? 0.f : m * c;
     float p[2][2];
     uint32_t ph[2], pm[2], pl[2];
 #pragma unroll
@@ -280,6 +280,23 @@ struct DecodeState {
     }
   }
 };
+
+// Element e of a head's output.  The three terms of a probability do not add up to an infinity when they multiply an
+// infinite value (a term may be zero or negative): a NaN whose weights are numbers is replaced by what the infinities
+// among the values say, and stays one where they are of both signs or a value is itself a NaN.
+template <int D>
+__device__ __forceinline__ float decode_output(float o, float l, const uint16_t* Vh, int n, int e) {
+  if (o == o || !(l < INFINITY)) return o;
+  bool pos = false, neg = false;
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const uint32_t w = Vh[(size_t)j * D + e];
+    if ((w & 0x7F80u) != 0x7F80u) continue;
+    if (w & 0x7Fu) return o;
+    (w >> 15 ? neg : pos) = true;
+  }
+  return pos == neg ? o : pos ? INFINITY : -INFINITY;
+}
 
 // GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
 // MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
@@ -451,8 +468,10 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
       }
       if (!MASS && a.n_groups == 1) {
         const float inv = ll > 0.f ? 1.f / ll : 0.f;
-        *reinterpret_cast<float4*>(a.out[layer] + (size_t)(h * G + g) * D + e0) =
-            make_float4(aa[0] * inv, aa[1] * inv, aa[2] * inv, aa[3] * inv);
+        float o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = decode_output<D>(aa[e] * inv, ll, Vh, n, e0 + e);
+        *reinterpret_cast<float4*>(a.out[layer] + (size_t)(h * G + g) * D + e0) = make_float4(o[0], o[1], o[2], o[3]);
       } else {
         float* dst = a.part + ((size_t)blockIdx.x * G + g) * (D + 4);
         if (e0 == 0) {
@@ -530,7 +549,9 @@ __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __
         const float v2[1] = {s_v[w][threadIdx.x]};
         merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
       }
-      a.out[layer][(size_t)(h * G + g) * D + threadIdx.x] = l1 > 0.f ? v1[0] / l1 : 0.f;
+      const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
+      a.out[layer][(size_t)(h * G + g) * D + threadIdx.x] =
+          decode_output<D>(l1 > 0.f ? v1[0] / l1 : 0.f, l1, Vh, max(0, min(decode_n(a), a.n_cap)), (int)threadIdx.x);
     }
     return;
   }

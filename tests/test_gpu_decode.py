@@ -132,6 +132,31 @@ def test_decode_stream_split(B, G, d, h2o, n):
         assert not mass[0][:, n:].any()
 
 
+@pytest.mark.parametrize("G", [4, 5])
+@pytest.mark.parametrize("Hkv,n", [(2, 60), (2, 3000), (64, 8190)])
+def test_decode_infinities(B, Hkv, n, G):
+    """Infinite values reach the output as infinities (both signs or a NaN among them: NaN), and keys whose logit is -inf,
+    48 in a row, weigh nothing: one CTA per pair, split pairs, and streamed ranges."""
+    import torch
+    d = 128
+    rng = np.random.default_rng(n + G)
+    q, K, V = _bits(rng, (Hkv * G, d), 2.0), _bits(rng, (Hkv, n, d)), _bits(rng, (Hkv, n, d))
+    q[:, 7] &= 0x7FFF                                   # positive
+    K[:, :48, 7] = 0xFF80                               # -inf
+    mask = np.ones(n, bool)
+    mask[:48] = False
+    want = O.decode_attention(q, K[:, mask], V[:, mask])
+    V[:, 50, 3], V[:, 52, 4], V[:, 54, 5], V[:, 55, 6] = 0x7F80, 0xFF80, 0x7F80, 0x7FC0
+    V[:, 53, 5] = 0xFF80
+    want[:, 3], want[:, 4], want[:, 5], want[:, 6] = np.inf, -np.inf, np.nan, np.nan
+    st = B.new_status()
+    out = B.stepkv_decode([TL.bf16_dev(q)], [TL.bf16_dev(K)], [TL.bf16_dev(V)], n, status=st)[0].cpu().numpy()
+    assert st.item() == 0
+    np.testing.assert_array_equal(out[:, 3:7], want[:, 3:7].astype(np.float32))
+    keep = [e for e in range(d) if not 3 <= e < 7]
+    assert np.abs(out[:, keep] - want[:, keep]).max() < 1e-5
+
+
 def test_decode_rejects_one_bad_layer_among_many(B):
     """Layers laid out alike are checked once: one that differs, wherever it stands, is still found."""
     import torch
