@@ -60,6 +60,7 @@ struct DecodeArgs {
   int n_groups;         // CTAs per pair (split form)
   int n_warps;          // warps of the launch (stream form), 0: split form
   int chunks;           // accumulated attention: blocks of the merge kernel per pair
+  int prefetch;         // split form: decode_prefetch before the wait
   const int32_t* n_dev;
   int n_host;
   int n_cap;
@@ -76,6 +77,11 @@ static_assert(sizeof(DecodeArgs) <= 32000, "kernel parameter space");
 __device__ __forceinline__ int decode_n(const DecodeArgs& a) {
   const int n = a.n_dev ? *a.n_dev : a.n_host;
   return n;
+}
+
+// Keys per CTA of the split form.
+__device__ __forceinline__ int decode_share(int n, int groups) {
+  return ((n + groups - 1) / groups + kDecBlock - 1) & ~(kDecBlock - 1);
 }
 
 // D = A B for one m16n8k16 tile of bf16 operands, from a zero accumulator.
@@ -298,6 +304,32 @@ __device__ __forceinline__ float decode_output(float o, float l, const uint16_t*
   return pos == neg ? o : pos ? INFINITY : -INFINITY;
 }
 
+// The last warp of a split-form CTA sends for the first 32 KB of the CTA's keys and of its values into L2 while the kernel
+// before it finishes: with a call per layer that is the merge of the layer before, which leaves DRAM idle for ~3 us.  L2
+// holds what memory holds, so rows still being written are read right after the wait; the number of keys may still
+// change, so here it only tells where the share probably lies.  8 heads x 8272 rows, calls in a row: 13.7 -> 13.0 us (64
+// KB or the whole share: no better), with another kernel between them 14.9 -> 15.0; 32 layers in a captured step 393 ->
+// 368 us.
+// Only where the CTAs fill half the machine and have more rows than their rings (else the reads are short, and the warp
+// that prefetches starts late: 1500 rows, 32 CTAs, another kernel between the calls 8.9 -> 9.3 us; 548 rows 5.9 -> 6.9),
+// and not with accumulated attention, whose mass blocks read in that gap (one layer 22.9 -> 24.4 us).
+constexpr int kDecPrefetchBytes = 32 << 10;
+template <int D>
+__device__ __forceinline__ void decode_prefetch(const DecodeArgs& a) {
+  constexpr int kPieces = 16;  // per tensor
+  const int t = (int)threadIdx.x - (kDecThreads - 2 * kPieces);
+  if (t < 0) return;
+  const int n = max(0, min(a.n_dev ? __ldcg(a.n_dev) : a.n_host, a.n_cap));  // (not through L1: read again after the wait)
+  const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
+  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
+  const int share = decode_share(n, a.n_groups);
+  const int k_begin = min(n, grp * share);
+  const int rows = min(min(n - k_begin, share), kDecPrefetchBytes / (2 * D));
+  const int per = (rows + kPieces - 1) / kPieces, r0 = min(rows, (t >> 1) * per), r1 = min(rows, r0 + per);
+  const uint16_t* base = ((t & 1) ? a.V[layer] : a.K[layer]) + (size_t)h * a.head_stride;
+  if (r1 > r0) bulk_prefetch_l2(base + (size_t)(k_begin + r0) * D, (uint32_t)(r1 - r0) * 2 * D);
+}
+
 // GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
 // MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
 // STREAM: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
@@ -311,6 +343,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
   constexpr int kStages = kDecRingBytes / kStageBytes;
   extern __shared__ __align__(16) uint8_t dec_smem[];     // per-warp rings | logits (MASS, cluster form)
 
+  if constexpr (!STREAM && !MASS)
+    if (a.prefetch) decode_prefetch<D>(a);
   pdl_wait();
   pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -427,7 +461,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
     __shared__ float s_ml[NW][GP][2];
     const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
     const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
-    const int share = ((n + a.n_groups - 1) / a.n_groups + kDecBlock - 1) & ~(kDecBlock - 1);
+    const int share = decode_share(n, a.n_groups);
     const int k_begin = min(n, grp * share), k_end = min(n, k_begin + share);
     const uint16_t* Kh = a.K[layer] + (size_t)h * a.head_stride;
     const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
@@ -599,7 +633,7 @@ size_t decode_mass_ws_bytes(int n_layers, int Hkv, int Hq, int d, int n_cap) {
 // How a launch splits `pairs` (layer, KV head) pairs of up to n_cap keys.  The stream form balances every SM and fills
 // its ring once, but a warp must have blocks enough to be worth a partial state, and the workspace holds
 // pairs x ceil(n_cap / 512) of them: it is taken where that allows three quarters of the machine's warps.  Else each pair
-// is split over as many CTAs as one wave and the workspace hold: one layer of 8 heads x 8272 rows takes 12.2 us per call
+// is split over as many CTAs as one wave and the workspace hold: one layer of 8 heads x 8272 rows takes 11.5 us per call
 // in a captured step (27.3 us with 512-key splits and 16-byte loads into registers; a cluster of 16 CTAs per pair with
 // the merge through distributed shared memory 24 us, since only 7 such clusters fit at a time; the last CTA of a pair
 // merging, found by an atomic count, 18.5 us).
@@ -674,6 +708,7 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
     a.pairs = nl * Hkv;
     a.n_groups = p.groups;
     a.n_warps = p.n_warps;
+    a.prefetch = 2 * a.pairs * p.groups >= n_sm && (int64_t)(n_cap / p.groups) * (4 * d) > kDecWarps * kDecRingBytes;
     a.chunks = std::max(1, std::min(8, (n_cap + 1023) / 1024));
     a.n_dev = n_dev;
     a.n_host = n_host;

@@ -132,6 +132,35 @@ def test_decode_stream_split(B, G, d, h2o, n):
         assert not mass[0][:, n:].any()
 
 
+@pytest.mark.parametrize("Hkv,d,rows", [(2, 128, 60), (2, 64, 600), (8, 128, 8911)])
+def test_decode_chain_with_changing_n(B, Hkv, d, rows):
+    """Calls in a row whose number of keys is written on the device just before each: a call that starts fetching while
+    its predecessor finishes sees an older count, above, below or out of range, and must not depend on it.  The rows past
+    n are NaN."""
+    import torch
+    rng = np.random.default_rng(rows)
+    q = TL.bf16_dev(_bits(rng, (Hkv * 4, d), 2.0))
+    ns = [rows, 1, rows // 2, 17, rows, 33, rows - 1, 16]
+    K, V = [], []
+    for n in ns:
+        for x in (K, V):
+            t = torch.full((Hkv, rows, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+            t[:, :n] = TL.bf16_dev(_bits(rng, (Hkv, n, d)))
+            x.append(t)
+    st, n_dev = B.new_status(), torch.full((1,), 2**31 - 1, dtype=torch.int32, device="cuda")
+    alone = [B.stepkv_decode([q], [k], [v], n, status=st)[0] for k, v, n in zip(K, V, ns)]
+    torch.cuda.synchronize()
+    chain = []
+    for k, v, n in zip(K, V, ns):
+        n_dev.fill_(n)
+        chain.append([B.stepkv_decode([q], [k], [v], n_dev, status=st)[0] for _ in range(3)])
+        n_dev.fill_(2**31 - 1)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    for want, got, n in zip(alone, chain, ns):
+        assert torch.isfinite(want).all() and all(torch.equal(g, want) for g in got), n
+
+
 @pytest.mark.parametrize("G", [4, 5])
 @pytest.mark.parametrize("Hkv,n", [(2, 60), (2, 3000), (64, 8190)])
 def test_decode_infinities(B, Hkv, n, G):
