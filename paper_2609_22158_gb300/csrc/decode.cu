@@ -74,9 +74,10 @@ struct DecodeArgs {
 
 static_assert(sizeof(DecodeArgs) <= 32000, "kernel parameter space");
 
-__device__ __forceinline__ int decode_n(const DecodeArgs& a) {
-  const int n = a.n_dev ? *a.n_dev : a.n_host;
-  return n;
+// early: before the wait (the count may still change, so it must not stay in L1).
+__device__ __forceinline__ int decode_n(const DecodeArgs& a, bool early = false) {
+  if (!a.n_dev) return a.n_host;
+  return early ? __ldcg(a.n_dev) : *a.n_dev;
 }
 
 // Keys per CTA of the split form.
@@ -309,7 +310,7 @@ __device__ __forceinline__ float decode_output(float o, float l, const uint16_t*
 // holds what memory holds, so rows still being written are read right after the wait; the number of keys may still
 // change, so here it only tells where the share probably lies.  8 heads x 8272 rows, calls in a row: 13.7 -> 13.0 us (64
 // KB or the whole share: no better), with another kernel between them 14.9 -> 15.0; 32 layers in a captured step 393 ->
-// 368 us.
+// 368 us (307 with the merge's dry run).
 // Only where the CTAs fill half the machine and have more rows than their rings (else the reads are short, and the warp
 // that prefetches starts late: 1500 rows, 32 CTAs, another kernel between the calls 8.9 -> 9.3 us; 548 rows 5.9 -> 6.9),
 // and not with accumulated attention, whose mass blocks read in that gap (one layer 22.9 -> 24.4 us).
@@ -319,7 +320,7 @@ __device__ __forceinline__ void decode_prefetch(const DecodeArgs& a) {
   constexpr int kPieces = 16;  // per tensor
   const int t = (int)threadIdx.x - (kDecThreads - 2 * kPieces);
   if (t < 0) return;
-  const int n = max(0, min(a.n_dev ? __ldcg(a.n_dev) : a.n_host, a.n_cap));  // (not through L1: read again after the wait)
+  const int n = max(0, min(decode_n(a, true), a.n_cap));
   const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
   const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
   const int share = decode_share(n, a.n_groups);
@@ -520,13 +521,13 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
 
 // The partial slots of a pair, in key order: of the stream form those of the warps whose ranges reach into the pair,
 // else its CTAs' (all of them, empty shares included, so that the number of keys need not be read first).
-__device__ __forceinline__ void decode_slots(const DecodeArgs& a, int pair, int& first, int& count) {
+__device__ __forceinline__ void decode_slots(const DecodeArgs& a, int pair, int& first, int& count, bool early = false) {
   if (a.n_warps == 0) {
     first = pair * a.n_groups;
     count = a.n_groups;
     return;
   }
-  const int n = max(0, min(decode_n(a), a.n_cap));
+  const int n = max(0, min(decode_n(a, early), a.n_cap));
   const int nb = (n + kDecBlock - 1) / kDecBlock;
   const int per = (a.pairs * nb + a.n_warps - 1) / a.n_warps;
   first = count = 0;
@@ -537,58 +538,85 @@ __device__ __forceinline__ void decode_slots(const DecodeArgs& a, int pair, int&
 }
 
 // Merge of the partial states.  Blocks [0, pairs * G) take one (pair, head) each: warp w merges slots w, w + 4, ... in
-// order (the loads of eight in flight), then the warps meet in order, and out = acc / l.  With accumulated attention,
+// order, then the warps meet in order, and out = acc / l.  With accumulated attention,
 // `chunks` more blocks per pair each take a contiguous share of the keys: the heads' log-sum-exp from all slots, then
 // the group-mean softmax mass of every key of the share is added (one writer per key).
+// A merge is a chain of latencies of code that runs once, and its blocks lie idle while the decode kernel works: so a
+// block first goes through it without its loads and its store (but for one load, for the address translation), which
+// brings in the code and the parameters, and only then waits.  And the loads of a warp's next four slots are in flight
+// before the first is merged.  One layer of 8 heads x 8272 rows, calls in a row: 13.0 -> 10.1 us, with another kernel
+// between them 15.0 -> 12.6; 4240 rows 10.3 -> 8.2; 2 heads x 16000 rows 9.2 -> 8.2; 8 layers 50.9 -> 48.5; 32 layers 168.8
+// -> 168.2.  (Eight slots: 9.7, but 8 query heads or fewer rows slower, 32 layers 170.5.  An unrolled loop left to the
+// compiler: 10.8-11.5, 2 heads up to 10.9.)  With accumulated attention the blocks are too many to lie idle (one layer
+// 22.6 -> 24.1 us with the dry run), so those wait at once.
 constexpr int kDecMergeThreads = 128;
 
-template <int D>
+template <int D, bool MASS>
 __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __grid_constant__ DecodeArgs a) {
-  constexpr int PER = D / 32, NW = kDecMergeThreads / 32;
+  constexpr int PER = D / 32, NW = kDecMergeThreads / 32, kSlotsInFlight = 4;
   __shared__ float s_ml[NW][2];
   __shared__ float s_v[NW][D];
   __shared__ float s_lse[8];
-  pdl_wait();
-  pdl_launch_dependents();
   const int G = a.G, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int item = (int)blockIdx.x;
   int first, count;
-  if (item < a.pairs * G) {
+  if (!MASS || item < a.pairs * G) {
     const int pair = item / G, g = item - pair * G;
     const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
-    decode_slots(a, pair, first, count);
-    float mm = -INFINITY, ll = 0.f, aa[PER];
-#pragma unroll
-    for (int e = 0; e < PER; ++e) aa[e] = 0.f;
-#pragma unroll 8
-    for (int i = warp; i < count; i += NW) {
-      const float* src = a.part + ((size_t)(first + i) * G + g) * (D + 4);
-      const float2 ml = __ldcg(reinterpret_cast<const float2*>(src));
-      float a2[PER];
-#pragma unroll
-      for (int e = 0; e < PER; ++e) a2[e] = __ldcg(src + 4 + e * 32 + lane);
-      merge_state<PER>(mm, ll, aa, ml.x, ml.y, a2);
-    }
-    if (lane == 0) {
-      s_ml[warp][0] = mm;
-      s_ml[warp][1] = ll;
-    }
-#pragma unroll
-    for (int e = 0; e < PER; ++e) s_v[warp][e * 32 + lane] = aa[e];
-    __syncthreads();
-    if ((int)threadIdx.x < D) {
-      float m1 = -INFINITY, l1 = 0.f, v1[1] = {0.f};
-#pragma unroll
-      for (int w = 0; w < NW; ++w) {
-        const float v2[1] = {s_v[w][threadIdx.x]};
-        merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
+#pragma unroll 1
+    for (int rep = MASS ? 1 : 0; rep < 2; ++rep) {
+      const bool live = MASS || rep == 1;
+      if (live) {
+        pdl_wait();
+        pdl_launch_dependents();
       }
-      const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
-      a.out[layer][(size_t)(h * G + g) * D + threadIdx.x] =
-          decode_output<D>(l1 > 0.f ? v1[0] / l1 : 0.f, l1, Vh, max(0, min(decode_n(a), a.n_cap)), (int)threadIdx.x);
+      decode_slots(a, pair, first, count, !live);
+      float mm = -INFINITY, ll = 0.f, aa[PER];
+#pragma unroll
+      for (int e = 0; e < PER; ++e) aa[e] = 0.f;
+      if (!live && lane == 0) s_ml[warp][0] = __ldcg(a.part);
+#pragma unroll 1
+      for (int i0 = warp; i0 < count; i0 += kSlotsInFlight * NW) {
+        float2 ml[kSlotsInFlight];
+        float a2[kSlotsInFlight][PER];
+#pragma unroll
+        for (int u = 0; u < kSlotsInFlight; ++u) {
+          const float* src = a.part + ((size_t)(first + i0 + u * NW) * G + g) * (D + 4);
+          const bool ok = live && i0 + u * NW < count;
+          ml[u] = ok ? __ldcg(reinterpret_cast<const float2*>(src)) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+          for (int e = 0; e < PER; ++e) a2[u][e] = ok ? __ldcg(src + 4 + e * 32 + lane) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kSlotsInFlight; ++u) merge_state<PER>(mm, ll, aa, ml[u].x, ml[u].y, a2[u]);
+      }
+      if (lane == 0) {
+        s_ml[warp][0] = mm;
+        s_ml[warp][1] = ll;
+      }
+#pragma unroll
+      for (int e = 0; e < PER; ++e) s_v[warp][e * 32 + lane] = aa[e];
+      __syncthreads();
+      if ((int)threadIdx.x < D) {
+        float m1 = -INFINITY, l1 = 0.f, v1[1] = {0.f};
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          const float v2[1] = {s_v[w][threadIdx.x]};
+          merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
+        }
+        float* out = a.out[layer] + (size_t)(h * G + g) * D + threadIdx.x;
+        const float o = l1 > 0.f ? v1[0] / l1 : 0.f;
+        if (live) {
+          const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
+          *out = decode_output<D>(o, l1, Vh, max(0, min(decode_n(a), a.n_cap)), (int)threadIdx.x);
+        }
+      }
+      __syncthreads();
     }
     return;
   }
+  pdl_wait();
+  pdl_launch_dependents();
   const int rest = item - a.pairs * G, pair = rest / a.chunks, chunk = rest - pair * a.chunks;
   const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
   decode_slots(a, pair, first, count);
@@ -633,7 +661,7 @@ size_t decode_mass_ws_bytes(int n_layers, int Hkv, int Hq, int d, int n_cap) {
 // How a launch splits `pairs` (layer, KV head) pairs of up to n_cap keys.  The stream form balances every SM and fills
 // its ring once, but a warp must have blocks enough to be worth a partial state, and the workspace holds
 // pairs x ceil(n_cap / 512) of them: it is taken where that allows three quarters of the machine's warps.  Else each pair
-// is split over as many CTAs as one wave and the workspace hold: one layer of 8 heads x 8272 rows takes 11.5 us per call
+// is split over as many CTAs as one wave and the workspace hold: one layer of 8 heads x 8272 rows takes 9.6 us per call
 // in a captured step (27.3 us with 512-key splits and 16-byte loads into registers; a cluster of 16 CTAs per pair with
 // the merge through distributed shared memory 24 us, since only 7 such clusters fit at a time; the last CTA of a pair
 // merging, found by an atomic count, 18.5 us).
@@ -658,11 +686,12 @@ static cudaError_t decode_launch(const DecodeArgs& a, cudaStream_t stream) {
   const int grid = STREAM ? a.n_warps / kDecWarps : a.pairs * a.n_groups;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), smem);
   // Both kernels launch dependently (each waits for the one before it before it reads anything): a captured decode
-  // step of 32 one-layer calls takes 390 us, 406 with the first launched plainly, 541 with both.
+  // step of 32 one-layer calls took 390 us when neither did anything before its wait, 406 with the first launched
+  // plainly, 541 with both; with the prefetch and the merge's dry run it takes 307.
   if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(kDecThreads), smem, stream, a, true);
   if (e != cudaSuccess || (!STREAM && !MASS && a.n_groups == 1)) return e;
   const int blocks = a.pairs * (a.G + (MASS ? a.chunks : 0));
-  return launch_kernel(decode_merge_kernel<D>, dim3(blocks), dim3(kDecMergeThreads), 0, stream, a, true);
+  return launch_kernel(decode_merge_kernel<D, MASS>, dim3(blocks), dim3(kDecMergeThreads), 0, stream, a, true);
 }
 
 template <int D, int GP>
