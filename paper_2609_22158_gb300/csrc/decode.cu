@@ -685,9 +685,9 @@ static cudaError_t decode_launch(const DecodeArgs& a, cudaStream_t stream) {
   const int smem = kDecWarps * kDecRingBytes;
   const int grid = STREAM ? a.n_warps / kDecWarps : a.pairs * a.n_groups;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), smem);
-  // Both kernels launch dependently (each waits for the one before it before it uses anything that may still be written): a captured decode
-  // step of 32 one-layer calls took 390 us when neither did anything before its wait, 406 with the first launched
-  // plainly, 541 with both; with the prefetch and the merge's dry run it takes 307.
+  // Both kernels launch dependently (each waits for the one before it before it uses anything that may still be
+  // written): a captured decode step of 32 one-layer calls took 390 us when neither did anything before its wait, 406
+  // with the first launched plainly, 541 with both; with the prefetch and the merge's dry run it takes 307.
   if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(kDecThreads), smem, stream, a, true);
   if (e != cudaSuccess || (!STREAM && !MASS && a.n_groups == 1)) return e;
   const int blocks = a.pairs * (a.G + (MASS ? a.chunks : 0));
