@@ -167,8 +167,8 @@ struct ScoreCfg {
   static constexpr int kTabOff = kQBytes + kStages * kStageBytes;     // float negoff[2][256] | int pw[2][256]
   static constexpr int kCombOff = kTabOff + 2 * 2 * kMaxRows * 4;    // | float comb[2 grp][2 parity][128]
   static constexpr int kBarOff = kCombOff + 2 * 2 * 128 * 4;
-  // k_full/k_empty per stage, q_full/q_empty, acc_full/acc_empty[2], epi[2], p1_flushed, comb_full[8]
-  static constexpr int kNumBars = 2 * kStages + 2 + 4 + 2 + 1 + 8;
+  // k_full/k_empty per stage, q_full/q_empty, acc_full/acc_empty[2], epi[2], p1_flushed, comb_full[16]
+  static constexpr int kNumBars = 2 * kStages + 2 + 4 + 2 + 1 + 16;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;                 // tmem base, abort flag
   static constexpr int kBytes = kMiscOff + 16;
   static constexpr int kDynSmem = kBytes + 1024;                          // + alignment slack
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
   uint64_t* acc_empty = acc_full + 2;  // [2]
   uint64_t* epi_bar = acc_empty + 2;   // [2], one per epilogue group
   uint64_t* p1_flushed = epi_bar + 2;  // every epilogue warp has written its pass-1 partials
-  uint64_t* comb_full = p1_flushed + 1;  // [2 grp][4 quarters]: the second warp's share of an item (rows output)
+  uint64_t* comb_full = p1_flushed + 1;  // [2 grp][2 slots][4 quarters]: the second warp's share of an item (rows output)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + Cfg::kMiscOff);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + Cfg::kMiscOff + 4);
 
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
       mbar_init(&epi_bar[b], kGroupWarps);
     }
     mbar_init(p1_flushed, kEpiWarps);
-    for (int i = 0; i < 8; ++i) mbar_init(&comb_full[i], 1);
+    for (int i = 0; i < 16; ++i) mbar_init(&comb_full[i], 1);
     *abort_flag = 0;
     mbar_fence_init();
   }
@@ -874,15 +874,19 @@ __global__ void __launch_bounds__(kThreads, 1) score_kernel(const __grid_constan
                                        l2_policy_evict_last());
         } else {
           // saliency rows: the group's two warps on this quarter combine in a fixed order.  The second hands its
-          // share over and goes on; the slot alternates between the group's items, and it cannot reach the item after
-          // next before the first has released that item's accumulator, which it does after this item's read.
-          float* comb = combf + (n_done & 1) * 128;
-          uint64_t* bar = comb_full + grp * 4 + q;
+          // share over and goes on; slots (a share and its barrier) alternate between the group's items.  The second
+          // can be one item ahead, no more: it cannot reach the item after next before the first has released the
+          // next item's accumulator, which it does after this item's wait and read.  So a slot's barrier is never two
+          // phases past the one waited for, which a parity wait could not tell from none (one barrier for both slots
+          // could be: the first releases this item's accumulator before it waits).
+          const int slot = n_done & 1;
+          float* comb = combf + slot * 128;
+          uint64_t* bar = comb_full + (grp * 2 + slot) * 4 + q;
           if (s2 == 1) {
             comb[q * 32 + lk] = acc;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar);
-          } else if (!(ok = mbar_wait(bar, (uint32_t)n_done & 1u, abort_flag))) {
+          } else if (!(ok = mbar_wait(bar, (uint32_t)(n_done >> 1) & 1u, abort_flag))) {
             break;
           }
           if (s2 == 0 && j < Tb) {

@@ -77,6 +77,27 @@ def test_score_split_window_masks(B, Hkv, G, d, T, W, lse):
     TL.assert_close(sal[0].cpu().numpy(), O.window_attention_saliency(k, q), "sal")
 
 
+@pytest.mark.parametrize("Hkv,G,d,T,W,nl", [(8, 2, 128, 32768, 8, 3), (8, 1, 64, 32768, 32, 2), (4, 5, 128, 32768, 8, 3)])
+@pytest.mark.parametrize("lse", [False, True])
+def test_score_rows_few_query_rows(B, Hkv, G, d, T, W, nl, lse):
+    """Saliency rows of units with at most 32 query rows (16, 32; 40 beside them), several tiles per CTA: the second warp of
+    a quarter has no columns of its own and runs ahead of the one that adds its share in.  Every row is compared, over
+    launches in a row."""
+    import torch
+    rng = np.random.default_rng(W + G + d)
+    base = _rand_bits(rng, (Hkv, T, d))
+    Ks = [np.roll(base, 977 * l, axis=1) for l in range(nl)]
+    Qs = [_rand_bits(rng, (Hkv * G, W, d)) for _ in range(nl)]
+    stats = [torch.from_numpy(O.window_row_lse(k, q).astype(np.float32)).cuda() for k, q in zip(Ks, Qs)] if lse else None
+    st, K, Q = B.new_status(), [TL.bf16_dev(k) for k in Ks], [TL.bf16_dev(q) for q in Qs]
+    sal = [B.stepkv_score(K, Q, T, status=st, lse=stats) for _ in range(8)]
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    assert all(torch.equal(s, sal[0]) for s in sal)
+    for l in range(nl):
+        TL.assert_close(sal[0][l].cpu().numpy(), O.window_attention_saliency(Ks[l], Qs[l]), f"sal layer {l}")
+
+
 @pytest.mark.parametrize("Hkv,G,d,T,W,nl", SCORE_CASES + [(1, 4, 128, 2500, 512, 1), (1, 5, 128, 3000, 1024, 1)])
 def test_score_with_prefill_lse_matches_oracle(B, Hkv, G, d, T, W, nl):
     """stepkv_score_lse: the rows' log-sum-exp comes from the caller (the oracle's, rounded to fp32, as
