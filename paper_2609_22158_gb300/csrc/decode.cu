@@ -714,9 +714,10 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
   }
   float* part = static_cast<float*>(ws);
   float* logits = nullptr;
-  if (mass != nullptr)
+  if (mass != nullptr)  // after one launch's partial states, as decode_mass_ws_bytes has it
     logits = reinterpret_cast<float*>(static_cast<uint8_t*>(ws) +
-                                      ((decode_ws_bytes(n_layers, Hkv, Hq, d, n_cap) + 255) & ~(size_t)255));
+                                      ((decode_ws_bytes(std::min(n_layers, kMaxDecodeLayers), Hkv, Hq, d, n_cap) + 255) &
+                                       ~(size_t)255));
   for (int l0 = 0; l0 < n_layers; l0 += kMaxDecodeLayers) {
     const int nl = std::min(kMaxDecodeLayers, n_layers - l0);
     DecodeArgs a;

@@ -68,6 +68,30 @@ def test_h2o_mass_matches_oracle(B, Hkv, G, d, n, rows, L, reads, ks):
         assert np.allclose(g[:, :n].sum(axis=1), reads, rtol=1e-5)
 
 
+@pytest.mark.parametrize("L", [64, 65, 80])
+def test_h2o_many_layers_stay_in_workspace(B, L):
+    """More layers than one launch takes: the launches share one workspace, sized for the largest, and nothing past it
+    is written.  Every layer's masses and outputs are compared."""
+    import torch
+    rng = np.random.default_rng(L)
+    Hkv, G, d, rows = 2, 4, 64, 600
+    some = [(_bits(rng, (Hkv * G, d)), _bits(rng, (Hkv, rows, d)), _bits(rng, (Hkv, rows, d))) for _ in range(7)]
+    dev = [tuple(TL.bf16_dev(x) for x in s) for s in some]
+    q, K, V = ([dev[l % 7][i] for l in range(L)] for i in range(3))
+    need = B.load_library().stepkv_decode_h2o_workspace_size(L, Hkv, Hkv * G, d, rows) + 256
+    buf = torch.full((need + (8 << 20),), 0xA5, dtype=torch.uint8, device="cuda")
+    mass = [torch.zeros((Hkv, rows), dtype=torch.float32, device="cuda") for _ in range(L)]
+    st = B.new_status()
+    out = B.stepkv_decode_h2o(q, K, V, rows, mass, ws=buf[:need], status=st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    assert (buf[need:] == 0xA5).all(), "written past the workspace"
+    for l in range(L):
+        ref = some[l % 7]
+        TL.assert_close(mass[l].cpu().numpy(), O.decode_attention_mass(ref[0], ref[1]), f"mass layer {l}", floor=1e-30)
+        TL.assert_decode_close(out[l].cpu().numpy(), *ref, f"layer {l}")
+
+
 def test_h2o_n_on_device_and_determinism(B):
     import torch
     rng = np.random.default_rng(8)
