@@ -140,6 +140,10 @@ struct ClusterOps {
   __device__ ClusterOps() : cluster(cg::this_cluster()) {}
   __device__ int rank() const { return (int)cluster.block_rank(); }
   __device__ void sync() { cluster.sync(); }
+  // Every thread of the kernel: started() once at its beginning, then all_started() before the first access to another
+  // CTA's shared memory, which exists only once that CTA runs.
+  __device__ void started() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+  __device__ void all_started() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
   template <typename P>
   __device__ P* peer(P* p, int r) { return cluster.map_shared_rank(p, r); }
 };
@@ -147,6 +151,8 @@ template <>
 struct ClusterOps<1> {
   __device__ int rank() const { return 0; }
   __device__ void sync() { __syncthreads(); }
+  __device__ void started() {}
+  __device__ void all_started() {}
   template <typename P>
   __device__ P* peer(P* p, int) { return p; }
 };
@@ -203,6 +209,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
   // Launched with programmatic dependent launch: everything up to pdl_wait() reads only the call's inputs and writes
   // only this kernel's workspace and outputs, so it may overlap the tail of the kernel that produces the saliency.
   pdl_launch_dependents();
+  cl.started();
   int lN = 0, lerr = 0;
 #pragma unroll 1
   for (int i0 = s0 + lane; i0 < s1; i0 += 32 * U) {
@@ -294,6 +301,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
     w_max[warp] = lmax;
     w_min[warp] = lmin;
   }
+  cl.all_started();  // the pushes below reach into every CTA (long since true: the tokens have been read meanwhile)
   __syncthreads();
   if (warp == 0) {
     float m = lane < NW ? w_max[lane] : -INFINITY, mi = lane < NW ? w_min[lane] : INFINITY;

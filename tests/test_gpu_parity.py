@@ -509,6 +509,31 @@ def test_select_large_T(B):
     TL.check_select_outputs(g, out)
 
 
+def test_select_clusters_side_by_side(B):
+    """More selections at once than clusters fit the machine, on streams of their own, so that a cluster's CTAs start while
+    others still run: each must agree with the oracle."""
+    import torch
+    tr = wl.custom(77, L=1, Hq=4, Hkv=1, d=64, T=2500, W=8, n_steps=9, budget=wl.Budget.ratio(1, 4))
+    sal = (np.random.default_rng(77).random((3, tr.T)) ** 3).astype(np.float32)
+    g, want, st = _select_case(B, tr, B.Params(), sal)
+    assert st == 0
+    TL.check_select_outputs(g, want)
+    sal, st = torch.from_numpy(sal).cuda(), B.new_status()
+    outs = [B.SelectOutputs.allocate(tr.T, tr.n_steps, tr.T, "cuda") for _ in range(96)]
+    streams = [torch.cuda.Stream() for _ in range(32)]
+    torch.cuda.synchronize()
+    for i, o in enumerate(outs):
+        with torch.cuda.stream(streams[i % len(streams)]):
+            steps = B.StepSignals(g.valid, g.gain, g.red, g.reuse_in, g.obs_sim)
+            B.stepkv_select(sal, g.step_id, g.prot, steps, B.Params(), B.budget_ratio(1, 4), o, status=st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    n = int(g.out.n_kept.item())
+    for o in outs:
+        assert int(o.n_kept.item()) == n and torch.equal(o.kept_idx[:n], g.out.kept_idx[:n])
+        assert torch.equal(o.step_kept, g.out.step_kept) and torch.equal(o.step_sal_sum, g.out.step_sal_sum)
+
+
 @pytest.mark.parametrize("n_steps", [2048, 2600])
 def test_select_many_steps(B, n_steps):
     """Thousands of reasoning steps (a few tokens each): per-step statistics, S_k and the selection."""
