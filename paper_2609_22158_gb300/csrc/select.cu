@@ -503,8 +503,9 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
       cl.sync();  // every CTA's histogram and coarse counts of this pass are complete
       if (warp == 0) {
         // The digit in two steps (keys in descending order): the coarse bin that holds the remaining-th largest key
-        // (lane l: coarse bins 8 l .. 8 l + 7), then the bin within it (lane l: fine bin l).
-        constexpr int PL = kCoarse / 32;
+        // (lane l: coarse bins PL l .. PL l + PL - 1), then the bin within it (lane l: fine bin l).
+        constexpr int PL = kCoarse / 32;  // 8, or 2 with 11 bits
+        static_assert(kCoarse % 64 == 0, "a lane's coarse counts are read in pairs");
         int cnt[PL];
 #pragma unroll
         for (int i = 0; i < PL; ++i) cnt[i] = 0;
@@ -512,11 +513,10 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
 #pragma unroll
           for (int r = 0; r < NC; ++r) {
 #pragma unroll
-            for (int i = 0; i < PL; i += 4) {
-              const int4 v = *reinterpret_cast<const int4*>(&ac[r * kCoarse + lane * PL + i]);
-              const int w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-              for (int x = 0; x < 4; ++x) cnt[i + x] += lane * PL + i + x < n_coarse ? w[x] : 0;
+            for (int i = 0; i < PL; i += 2) {
+              const int2 v = *reinterpret_cast<const int2*>(&ac[r * kCoarse + lane * PL + i]);
+              cnt[i] += lane * PL + i < n_coarse ? v.x : 0;
+              cnt[i + 1] += lane * PL + i + 1 < n_coarse ? v.y : 0;
             }
           }
         }

@@ -509,6 +509,30 @@ def test_select_large_T(B):
     TL.check_select_outputs(g, out)
 
 
+@pytest.mark.parametrize("T", [197900, 198000, 262144])
+@pytest.mark.parametrize("kind", ["cube", "ties", "rising"])
+def test_select_largest_T(B, kind, T):
+    """Around the length where the digits go from 13 to 11 bits, and the largest length: thresholds in the last and the
+    first bins, and thousands of tied priorities.  Exact at every budget (alpha = 1, beta = 0: the fp32 values rank)."""
+    import torch
+    rng = np.random.default_rng(T)
+    sal = {"cube": rng.random(T) ** 3, "ties": rng.integers(0, 9, T) / 8.0, "rising": np.arange(T) / T}[kind].astype(np.float32)
+    prot = np.zeros(T, np.uint8)
+    prot[:8], prot[-64:] = 1, 1
+    step_id = torch.from_numpy((np.arange(T) // 4096).astype(np.int32)).cuda()
+    z = lambda: torch.zeros(T // 4096 + 1, device="cuda")
+    steps = B.StepSignals(z(), z(), z(), z())
+    prunable = np.flatnonzero(prot == 0)
+    order = prunable[np.argsort(-sal[prunable], kind="stable")]
+    for count in (1, 8192, T // 2, T - 73):
+        out, st = B.SelectOutputs.allocate(T, T // 4096 + 1, T, "cuda"), B.new_status()
+        B.stepkv_select(torch.from_numpy(sal[None]).cuda(), step_id, torch.from_numpy(prot).cuda(), steps,
+                        B.Params(alpha=1.0, beta=0.0, sal_norm=B.NORM_NONE), B.budget_count(count), out, status=st)
+        assert int(st.item()) == 0
+        want = np.sort(np.concatenate([np.flatnonzero(prot), order[:count]]))
+        assert np.array_equal(out.kept_idx[:int(out.n_kept.item())].cpu().numpy(), want), (kind, T, count)
+
+
 def test_select_clusters_side_by_side(B):
     """More selections at once than clusters fit the machine, on streams of their own, so that a cluster's CTAs start while
     others still run: each must agree with the oracle."""
