@@ -412,6 +412,43 @@ def test_select_digits(B, kind, T):
         assert np.array_equal(gk, want), (kind, T, count)
 
 
+@pytest.mark.parametrize("T", [2000, 5000, 200000])
+@pytest.mark.parametrize("m", [1, 2, 255, 256, 257, 700])
+@pytest.mark.parametrize("beta", [0.0, 0.9])
+def test_select_few_keys_in_play(B, beta, m, T):
+    """m tokens, neighbouring floats or ties, share the threshold's bin of the first digit (one of the key, or linear
+    where the step utilities spread the priorities): up to 256 are ranked directly, more take further digits.  Thresholds at
+    the group's first, middle and last token and beside it; the order is that of the fp32 priorities the call reports."""
+    import torch
+    rng = np.random.default_rng(T + m)
+    n_steps = 6
+    step = np.sort(rng.integers(0, n_steps, T)).astype(np.int32)
+    sal = np.exp(rng.uniform(-12.0, 0.0, T)).astype(np.float32)
+    prot = np.zeros(T, np.uint8)
+    prot[:5], prot[-7:] = 1, 1
+    prunable = np.flatnonzero(prot == 0)
+    group = rng.permutation(prunable if beta == 0 else prunable[step[prunable] == 3][:10 * m + 10])[:m]
+    group = group if len(group) == m else rng.permutation(prunable)[:m]
+    sal[group] = np.float32(0.37) + rng.integers(0, max(1, m // 3), m).astype(np.float32) * np.float32(2.0**-25)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    zero = torch.zeros(n_steps, device="cuda")
+    steps = B.StepSignals(t(np.linspace(0.1, 1.0, n_steps).astype(np.float32)), zero, zero, zero)
+    p = B.Params(alpha=1.0 if beta == 0 else 0.01, beta=beta, sal_norm=B.NORM_NONE)
+    pri = None
+    for at in (None, -1, 0, 1, m // 2, m - 1, m):
+        if at is not None:
+            rank = prunable[np.argsort(-pri[prunable], kind="stable")]
+            first = int(np.flatnonzero(rank == group[np.argmax(pri[group])])[0])
+        count = T // 2 if at is None else max(1, first + at)
+        out, st = B.SelectOutputs.allocate(T, n_steps, T, "cuda"), B.new_status()
+        B.stepkv_select(t(sal[None]), t(step), t(prot), steps, p, B.budget_count(count), out, status=st)
+        assert int(st.item()) == 0
+        pri = out.priority.cpu().numpy()
+        order = prunable[np.argsort(-pri[prunable], kind="stable")]
+        want = np.sort(np.concatenate([np.flatnonzero(prot), order[:count]]))
+        assert np.array_equal(out.kept_idx[:int(out.n_kept.item())].cpu().numpy(), want), (at, count)
+
+
 @pytest.mark.parametrize("T", [1000, 9000])
 @pytest.mark.parametrize("kind", ["nan", "inf", "both", "all_nan", "overflow"])
 def test_select_non_finite_saliency(B, kind, T):
