@@ -110,12 +110,16 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t&
   lo = bf16x2_rn(x, y);
 }
 
-// Merge the state (m2, l2, acc2) into (m, l, acc), m in log2 units; -inf marks an empty state.
+// Merge the state (m2, l2, acc2) into (m, l, acc), m in log2 units; -inf marks an empty state (or one whose logits are all
+// NaN: its sum is NaN, and stays).
 template <int E>
 __device__ __forceinline__ void merge_state(float& m, float& l, float (&acc)[E], float m2, float l2,
                                             const float (&acc2)[E]) {
   const float mn = fmaxf(m, m2);
-  if (mn == -INFINITY) return;
+  if (mn == -INFINITY) {
+    l += l2;
+    return;
+  }
   const float a = ex2_approx(m - mn), b = ex2_approx(m2 - mn);
   l = l * a + l2 * b;
 #pragma unroll
@@ -502,7 +506,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
         merge_state<4>(mm, ll, aa, s_ml[w][g][0], s_ml[w][g][1], a2);
       }
       if (!MASS && a.n_groups == 1) {
-        const float inv = ll > 0.f ? 1.f / ll : 0.f;
+        const float inv = ll > 0.f ? 1.f / ll : ll;  // ll: 0 without keys, NaN where a logit is one (or +inf)
         float o[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[e] = decode_output<D>(aa[e] * inv, ll, Vh, n, e0 + e);
@@ -605,7 +609,7 @@ __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __
           merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
         }
         float* out = a.out[layer] + (size_t)(h * G + g) * D + threadIdx.x;
-        const float o = l1 > 0.f ? v1[0] / l1 : 0.f;
+        const float o = l1 > 0.f ? v1[0] / l1 : v1[0] * l1;  // l1: 0 without keys, NaN where a logit is one (or +inf)
         if (live) {
           const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
           *out = decode_output<D>(o, l1, Vh, max(0, min(decode_n(a), a.n_cap)), (int)threadIdx.x);

@@ -186,6 +186,36 @@ def test_decode_infinities(B, Hkv, n, G):
     assert np.abs(out[:, keep] - want[:, keep]).max() < 1e-5
 
 
+@pytest.mark.parametrize("kind", ["nan key", "inf logit", "only nan keys"])
+@pytest.mark.parametrize("G", [4, 5])
+@pytest.mark.parametrize("Hkv,n", [(2, 60), (2, 3000), (64, 8190)])
+def test_decode_nan_logits_reach_the_output(B, Hkv, n, G, kind):
+    """A key that is NaN, or a logit of +inf, makes every output of its KV head's query heads NaN: one CTA per pair, split
+    pairs, and streamed ranges, with and without accumulated attention.  The other heads are untouched."""
+    import torch
+    d = 128
+    rng = np.random.default_rng(n + G)
+    q, K, V = _bits(rng, (Hkv * G, d), 2.0), _bits(rng, (Hkv, n, d)), _bits(rng, (Hkv, n, d))
+    h = Hkv - 1
+    if kind == "nan key":
+        K[h, n // 2, 9] = 0x7FC0
+    elif kind == "inf logit":
+        q[h * G:, 9] &= 0x7FFF
+        K[h, n // 2, 9] = 0x7F80
+    else:
+        K[h, :, 9] = 0x7FC0
+    want = O.decode_attention(q[:h * G], K[:h], V[:h])
+    st = B.new_status()
+    args = [TL.bf16_dev(q)], [TL.bf16_dev(K)], [TL.bf16_dev(V)], n
+    mass = [torch.zeros((Hkv, n), dtype=torch.float32, device="cuda")]
+    for out in (B.stepkv_decode(*args, status=st)[0], B.stepkv_decode_h2o(*args, mass, status=st)[0]):
+        out = out.cpu().numpy()
+        assert st.item() == 0
+        assert np.isnan(out[h * G:]).all()
+        assert np.abs(out[:h * G] - want).max() < 1e-5
+    assert torch.isfinite(mass[0][:h]).all()
+
+
 def test_decode_rejects_one_bad_layer_among_many(B):
     """Layers laid out alike are checked once: one that differs, wherever it stands, is still found."""
     import torch
