@@ -110,16 +110,12 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t&
   lo = bf16x2_rn(x, y);
 }
 
-// Merge the state (m2, l2, acc2) into (m, l, acc), m in log2 units; -inf marks an empty state (or one whose logits are all
-// NaN: its sum is NaN, and stays).
+// Merge the state (m2, l2, acc2) into (m, l, acc), m in log2 units; -inf marks an empty state.
 template <int E>
 __device__ __forceinline__ void merge_state(float& m, float& l, float (&acc)[E], float m2, float l2,
                                             const float (&acc2)[E]) {
   const float mn = fmaxf(m, m2);
-  if (mn == -INFINITY) {
-    l += l2;
-    return;
-  }
+  if (mn == -INFINITY) return;
   const float a = ex2_approx(m - mn), b = ex2_approx(m2 - mn);
   l = l * a + l2 * b;
 #pragma unroll
@@ -286,7 +282,7 @@ struct DecodeState {
       }
     }
     if (writes && c4 == 0) {
-      ml[head * ml_stride] = m * c;
+      ml[head * ml_stride] = ls == ls ? m * c : INFINITY;  // a NaN sum is not to be merged as an empty state (all logits NaN)
       ml[head * ml_stride + 1] = ls;
     }
   }
