@@ -288,6 +288,10 @@ struct DecodeState {
   }
 };
 
+// A head's weighted value over its sum l: 0 without keys (l = 0), NaN where a logit is one or +inf (l is NaN).  The one
+// expression of every form: the output is the same bit for bit with and without accumulated attention.
+__device__ __forceinline__ float decode_quotient(float v, float l) { return l > 0.f ? v / l : v * l; }
+
 // Element e of a head's output.  The three terms of a probability do not add up to an infinity when they multiply an
 // infinite value (a term may be zero or negative): a NaN whose weights are numbers is replaced by what the infinities
 // among the values say, and stays one where they are of both signs or a value is itself a NaN.
@@ -502,10 +506,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
         merge_state<4>(mm, ll, aa, s_ml[w][g][0], s_ml[w][g][1], a2);
       }
       if (!MASS && a.n_groups == 1) {
-        const float inv = ll > 0.f ? 1.f / ll : ll;  // ll: 0 without keys, NaN where a logit is one (or +inf)
         float o[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) o[e] = decode_output<D>(aa[e] * inv, ll, Vh, n, e0 + e);
+        for (int e = 0; e < 4; ++e) o[e] = decode_output<D>(decode_quotient(aa[e], ll), ll, Vh, n, e0 + e);
         *reinterpret_cast<float4*>(a.out[layer] + (size_t)(h * G + g) * D + e0) = make_float4(o[0], o[1], o[2], o[3]);
       } else {
         float* dst = a.part + ((size_t)blockIdx.x * G + g) * (D + 4);
@@ -605,7 +608,7 @@ __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __
           merge_state<1>(m1, l1, v1, s_ml[w][0], s_ml[w][1], v2);
         }
         float* out = a.out[layer] + (size_t)(h * G + g) * D + threadIdx.x;
-        const float o = l1 > 0.f ? v1[0] / l1 : v1[0] * l1;  // l1: 0 without keys, NaN where a logit is one (or +inf)
+        const float o = decode_quotient(v1[0], l1);
         if (live) {
           const uint16_t* Vh = a.V[layer] + (size_t)h * a.head_stride;
           *out = decode_output<D>(o, l1, Vh, max(0, min(decode_n(a), a.n_cap)), (int)threadIdx.x);

@@ -68,6 +68,27 @@ def test_h2o_mass_matches_oracle(B, Hkv, G, d, n, rows, L, reads, ks):
         assert np.allclose(g[:, :n].sum(axis=1), reads, rtol=1e-5)
 
 
+@pytest.mark.parametrize("L,Hkv,G,d,n,rows", [(1, 2, 4, 128, 300, 300), (1, 2, 5, 64, 511, 512), (32, 8, 4, 128, 1500, 1500),
+                                              (10, 8, 8, 128, 700, 900), (25, 8, 1, 64, 333, 2000), (4, 8, 4, 128, 2500, 2500),
+                                              (32, 8, 2, 64, 3000, 6000)])
+def test_h2o_outputs_are_stepkv_decodes_bits(B, L, Hkv, G, d, n, rows):
+    """One CTA per pair (few rows, or more than half as many pairs as SMs), split pairs, and streamed ranges: the output is
+    the same bit for bit with and without accumulated attention."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(n + L)
+    rnd = lambda *s: [torch.randn(s, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(L)]
+    q, K, V = rnd(Hkv * G, d), rnd(Hkv, rows, d), rnd(Hkv, rows, d)
+    mass = [torch.zeros((Hkv, rows), dtype=torch.float32, device="cuda") for _ in range(L)]
+    st = B.new_status()
+    plain = B.stepkv_decode(q, K, V, n, status=st)
+    out = B.stepkv_decode_h2o(q, K, V, n, mass, status=st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    for l in range(L):
+        assert torch.equal(out[l], plain[l]), l
+        assert torch.allclose(mass[l].sum(1), torch.ones(Hkv, device="cuda"), rtol=1e-5)
+
+
 @pytest.mark.parametrize("L", [64, 65, 80])
 def test_h2o_many_layers_stay_in_workspace(B, L):
     """More layers than one launch takes: the launches share one workspace, sized for the largest, and nothing past it
