@@ -249,7 +249,8 @@ STEPKV_API stepkv_status_t stepkv_score_lse(int32_t n_layers, const void* const*
  *  prot      [T] uint8: 1 = protected.
  *  steps, params, budget: host structs (device arrays inside steps).
  *  out       host struct of device output pointers (see stepkv_select_out_t).
- *  Ranking: (P_i descending, slot index ascending) -- on equal priority the older token wins.
+ *  Ranking: (P_i descending, slot index ascending) -- on equal priority the older token wins.  A priority that is NaN
+ *           ranks below every number, -inf included.
  *  Supported: 1 <= T <= 262144, 1 <= n_steps <= 65535, n_sal >= 1.
  */
 STEPKV_API size_t stepkv_select_workspace_size(int32_t n_sal, int32_t T, int32_t n_steps);

@@ -338,7 +338,8 @@ __device__ __forceinline__ void decode_prefetch(const DecodeArgs& a) {
 // GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
 // MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
 // STREAM: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
-// per pair it touches (slot warp + pair); a merge kernel follows.  Else a cluster works on one pair.
+// per pair it touches (slot warp + pair).  Else (split form) n_groups CTAs of their own work on each pair and leave a partial
+// state each.  A merge kernel joins the states, but for plain reads with one CTA per pair, which write the output.
 template <int D, int GP, bool MASS, bool STREAM>
 __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_constant__ DecodeArgs a) {
   using State = DecodeState<D, GP>;
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
   constexpr int NCH = State::NCH;
   constexpr int kStageBytes = 2 * kDecBlock * D * 2;
   constexpr int kStages = kDecRingBytes / kStageBytes;
-  extern __shared__ __align__(16) uint8_t dec_smem[];     // per-warp rings | logits (MASS, cluster form)
+  extern __shared__ __align__(16) uint8_t dec_smem[];     // per-warp rings
 
   if constexpr (!STREAM && !MASS)
     if (a.prefetch) decode_prefetch<D>(a);
