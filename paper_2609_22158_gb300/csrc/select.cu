@@ -34,9 +34,6 @@ constexpr int kSelSingleMaxT = 2048;
 constexpr int kSelClusterCtas = 8;
 constexpr int kSelThreads = 1024;
 constexpr uint32_t kNanKey = 0x007FFFFEu;  // just below the key of -inf
-constexpr int kFewKeys = 256;              // keys of the threshold's bin that are ranked directly where digits would take
-constexpr int kFewKeysOneDigit = 64;       // two passes, or one
-constexpr int kNarrowBits = 16;            // more keys than that: bits undecided from which on their range is looked at
 
 struct SelectArgs {
   const float* T_in;                  // token saliency as floats, or
@@ -73,16 +70,6 @@ struct SelSummary {
   int n;               // prunable tokens
   int err;
 };
-
-// Zeroed with the histograms.  not_*: complements, whose zero means none.
-struct SelZeroed {
-  uint32_t not_lo, hi;  // range of this CTA's keys in play
-  int n_few;            // this CTA's keys handed to all
-  uint32_t not_kth;     // the threshold found by ranking, and how many ties of it are kept
-  int need_eq;
-};
-constexpr int kZeroedInts = 8;
-static_assert(sizeof(SelZeroed) <= kZeroedInts * 4, "SelZeroed");
 
 // Several independent trajectories in one launch: cluster (or CTA) c selects for trajectory c, so the
 // latency-bound passes of different trajectories run side by side on different SMs.
@@ -174,17 +161,18 @@ struct ClusterOps<1> {
 // launch and is fetched cold (so loops stay rolled).  There are as few of each as
 // the result allows:
 //  - the first digit is a linear bin of the priority between its bounds (the corners of alpha T^ + beta S over the
-//    extreme T^ and S), so the bins spread over the values the trajectory has.  Where the step utilities spread it by less
-//    than a 16th of what the saliency does, it is the leading digit of the key's offset from the lowest: the saliency is
-//    heavy-tailed, and with linear bins a selection by it alone (log-normal, all outputs) took up to five passes, 18.0 us
-//    at T = 2049 and 20.0 at 9000 (14.0 and 15.8 with key digits; three fixed digits 14.9 and 17.8).  Linear bins are the
-//    better ones at alpha = 0.8, beta = 0.2 (saliencies over 30 decades, T = 32768: 23.4 us; key digits 26.8);
-//  - the keys left in the threshold's bin are ranked directly where they are few, in one exchange: up to 64, or 256 where
-//    two more digits would be needed (the default weights, no statistics, T = 2049: 12.0 -> 11.3 us, T = 9000: 13.2 ->
-//    12.7; 75 ties: 0.3 us behind a digit, 50: level).  Else further digits of the key's offset follow; where more than
-//    256 keys and 16 bits are left, mostly ties, the digits that all of them share are skipped (saliencies of 0 and 1
-//    alone, T = 9000: 20.7 -> 15.9 us).  Three passes remain where the saliency rules and hundreds of tokens of a step
-//    nearly tie (alpha = 0.8, one outlier, T = 32768: 24.5 us; three fixed digits 22.2);
+//    extreme T^ and S), so the bins spread over the values the trajectory has; the keys of the threshold's bin span about
+//    BITS bits, and one more pass over the key's offset within the bin ranks them exactly (further passes where the bin
+//    reaches down to where floats are dense).  Fixed digits of the key took three passes, the first of which only told
+//    a few exponents apart.  Where the step utilities spread the priority by less than a 16th of what the saliency does, the
+//    passes begin with the leading digit of the key's offset from the lowest: the saliency is heavy-tailed, and with linear
+//    bins a selection by it alone (log-normal, all outputs) took up to five passes, T = 2049 / 9000 / 32768: 17.1 / 20.9 /
+//    25.0 us; with key digits 11.6 / 15.2 / 17.8 (fixed digits 14.0 / 19.1 / 24.1).  Linear bins are the better ones from
+//    there on (alpha = 0.8, beta = 0.2, saliencies over 30 decades, T = 32768: 23.4 us; key digits 26.8);
+//  - the passes end where all keys left in the threshold's bin are kept, mostly one key: two or three digits of a priority
+//    say no more than which tokens stay.  Ranking a few keys directly in one exchange instead of a last digit was up to
+//    0.8 us ahead where the code was warm, but its code costs a fused pass 2-4 us (T = 32768: 256.7 -> 260.7 us, 258.4
+//    where it is not even run);
 //  - every exchange is a push into the other CTAs' shared memory before a cluster barrier, so only the 32 fine counts
 //    of each digit are fetched after one;
 //  - a CTA's output offset comes out of the same counts (those of the CTAs before it above each digit), so no
@@ -202,11 +190,10 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
   ClusterOps<NC> cl;
   const int rank = cl.rank();
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  // layout: [2][kBins] int histograms | SelZeroed | [2][NC][kCoarse] every CTA's coarse counts | [chunk] T, then the ordered key of
+  // layout: [2][kBins] int histograms | [2][NC][kCoarse] every CTA's coarse counts | [chunk] T, then the ordered key of
   // P | [chunk] u16 step id (0xFFFF = protected) | S_k (when s_in_smem).  A token's entries are touched by one thread only.
   int* hist = reinterpret_cast<int*>(smem_raw);
-  SelZeroed* zeroed = reinterpret_cast<SelZeroed*>(hist + 2 * kBins);
-  int* coarse = hist + 2 * kBins + kZeroedInts;
+  int* coarse = hist + 2 * kBins;
   uint32_t* sKey = reinterpret_cast<uint32_t*>(coarse + 2 * NC * kCoarse);
   float* sT = reinterpret_cast<float*>(sKey);
   uint16_t* sSid = reinterpret_cast<uint16_t*>(sKey + a.chunk);
@@ -214,7 +201,6 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
   __shared__ SelSummary all[NC];
   __shared__ float w_max[NW], w_min[NW], s_lo[NW], s_hi[NW];
   __shared__ int w_n[NW], w_err[NW], w_strict[NW], w_eq[NW], bcast[5];
-  __shared__ uint2 ranges[NC];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int T = a.T, n_steps = a.steps.n_steps, t_last = n_steps - 1;
@@ -257,7 +243,7 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
     }
   }
 #pragma unroll 1
-  for (int i = tid; i < (2 * kBins + kZeroedInts) / 4; i += NT) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < 2 * kBins / 4; i += NT) reinterpret_cast<int4*>(hist)[i] = make_int4(0, 0, 0, 0);
   // Phases 1 and 2 of Algorithm 1 (Eqs. 2-4).  Every CTA computes all S_k, for their bounds and, where they fit, into
   // shared memory; CTA 0 publishes them.
   float b_lo = INFINITY, b_hi = -INFINITY;  // bounds of beta S_k
@@ -476,10 +462,6 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
     // keys as offsets from k_lo (one below the lowest: kNanKey below -inf), `left` bits of the threshold's undecided
     uint32_t k_lo = float_to_ordered(P_lo) - 1u, k_hi = float_to_ordered(P_hi) + 1u, prefix = 0u;
     int left = 32 - __clz((int)(k_hi - k_lo));
-    auto key_in_play = [&](uint32_t key) {
-      return first_bin(key) == star && (left >= 32 || ((key - k_lo) >> left) == prefix);
-    };
-    bool narrowed = false;
     const int first_pass = scale > 0.f ? 0 : 1;
 #pragma unroll 1
     for (int pass = first_pass;; ++pass) {
@@ -623,89 +605,14 @@ __global__ void __launch_bounds__(NT, 1) select_kernel(const __grid_constant__ S
         need_eq = remaining;
         break;
       }
-      if (in_bin > (left > BITS ? kFewKeys : kFewKeysOneDigit)) {
-        if (left < kNarrowBits || narrowed) continue;
-        // Many keys, and several digits to go: mostly ties, so the digits that all keys in play share are skipped.
-        narrowed = true;
-        uint32_t lo = 0xFFFFFFFFu, hi = 0u;  // offsets
-#pragma unroll 1
-        for (int i = s0 + lane; i < s1; i += 32) {
-          const uint32_t key = sKey[i];
-          if (sSid[i] != 0xFFFF && key_in_play(key)) {
-            lo = min(lo, key - k_lo);
-            hi = max(hi, key - k_lo);
-          }
-        }
-        lo = __reduce_min_sync(full, lo);
-        hi = __reduce_max_sync(full, hi);
-        if (lane == 0 && lo <= hi) {
-          atomicMax(&zeroed->not_lo, ~lo);
-          atomicMax(&zeroed->hi, hi);
-        }
-        __syncthreads();
-        if (tid < NC) *cl.peer(&ranges[rank], tid) = make_uint2(zeroed->not_lo, zeroed->hi);
-        cl.sync();
-        uint32_t not_lo = 0u;
-        hi = 0u;
-#pragma unroll
-        for (int r = 0; r < NC; ++r) {
-          not_lo = max(not_lo, ranges[r].x);
-          hi = max(hi, ranges[r].y);
-        }
-        left = 32 - __clz((int)(~not_lo ^ hi));
-        prefix = left < 32 ? hi >> left : 0u;
-        if (left > 0) continue;
-        kth = k_lo + prefix;
-        need_eq = remaining;
+      // All keys of the bin are kept (mostly it is one key): they lie above its lower bound less one, which the undecided
+      // bits do not change, if no key outside the linear bin does.
+      if (in_bin == remaining && pass > 0 && first_bin(k_lo + (prefix << left)) == star) {
+        kth = k_lo + (prefix << left) - 1u;
+        strict_pre += eq_pre;
+        eq_pre = 0;
         break;
       }
-      // Few keys in play: every CTA gets them all, in CTA order (eq_pre of them lie in the CTAs before this one; the
-      // coarse counts of the pass before are no longer read), and a warp ranks each among the others.
-      uint32_t* few = reinterpret_cast<uint32_t*>(coarse + ((pass + 1) & 1) * NC * kCoarse);
-#pragma unroll 1
-      for (int i0 = s0; i0 < s1; i0 += 32) {
-        const int i = i0 + lane;
-        const uint32_t key = i < s1 ? sKey[i] : 0u;
-        const bool hit = i < s1 && sSid[i] != 0xFFFF && key_in_play(key);
-        const unsigned hm = __ballot_sync(full, hit);
-        if (hm == 0u) continue;
-        int at = 0;
-        if (lane == 0) at = atomicAdd(&zeroed->n_few, __popc(hm));
-        at = eq_pre + __shfl_sync(full, at, 0) + __popc(hm & lt);
-        if (hit && at < kFewKeys) {
-#pragma unroll
-          for (int r = 0; r < NC; ++r) cl.peer(few, r)[at] = key;
-        }
-      }
-      cl.sync();
-      constexpr int kPerLane = kFewKeys / 32;
-      uint32_t in_play[kPerLane];
-#pragma unroll
-      for (int u = 0; u < kPerLane; ++u) in_play[u] = 32 * u + lane < in_bin ? few[32 * u + lane] : 0u;  // (no key is 0)
-#pragma unroll 1
-      for (int i = warp; i < in_bin; i += NW) {
-        const uint32_t key = few[i];
-        int n = 0;  // keys above this one, and in the upper half those that equal it
-#pragma unroll
-        for (int u = 0; u < kPerLane; ++u) n += in_play[u] > key ? 1 : in_play[u] == key ? 1 << 16 : 0;
-        n = __reduce_add_sync(full, n);
-        const int above = n & 0xFFFF;
-        if (lane == 0 && above < remaining && remaining <= above + (n >> 16)) {  // the threshold (ties write the same)
-          zeroed->not_kth = ~key;
-          zeroed->need_eq = remaining - above;
-        }
-      }
-      __syncthreads();
-      kth = ~zeroed->not_kth;
-      need_eq = zeroed->need_eq;
-      int n = 0;  // of the CTAs before this one
-#pragma unroll
-      for (int u = 0; u < kPerLane; ++u)
-        if (32 * u + lane < eq_pre) n += in_play[u] > kth ? 1 : in_play[u] == kth ? 1 << 16 : 0;
-      n = __reduce_add_sync(full, n);
-      strict_pre += n & 0xFFFF;
-      eq_pre = n >> 16;
-      break;
     }
   }
   if (B == 0 || B == N) copy_metadata(0);
@@ -947,7 +854,7 @@ static SelectArgs make_select_args(const SelectSpec& sp) {
 constexpr size_t kSelSmemMax = 232448 - 2048;
 static size_t select_smem(int chunk, int nc, int bits, int n_steps, int* s_in_smem) {
   const size_t bins = (size_t)1 << bits;
-  const size_t fixed = (2 * bins + kZeroedInts + 2 * nc * (bins / 32)) * 4 + (size_t)chunk * 6;
+  const size_t fixed = (2 * bins + 2 * nc * (bins / 32)) * 4 + (size_t)chunk * 6;
   *s_in_smem = fixed + (size_t)n_steps * 4 <= kSelSmemMax ? 1 : 0;
   return fixed + (*s_in_smem ? (size_t)n_steps * 4 : 0);
 }

@@ -415,9 +415,9 @@ def test_select_digits(B, kind, T):
 @pytest.mark.parametrize("T", [2000, 5000, 200000])
 @pytest.mark.parametrize("m", [1, 2, 255, 256, 257, 700])
 @pytest.mark.parametrize("beta", [0.0, 0.9])
-def test_select_few_keys_in_play(B, beta, m, T):
+def test_select_keys_in_the_thresholds_bin(B, beta, m, T):
     """m tokens, neighbouring floats or ties, share the threshold's bin of the first digit (one of the key, or linear
-    where the step utilities spread the priorities): up to 256 are ranked directly, more take further digits.  Thresholds at
+    where the step utilities spread the priorities): the passes end early where the bin's keys are all kept.  Thresholds at
     the group's first, middle and last token and beside it; the order is that of the fp32 priorities the call reports."""
     import torch
     rng = np.random.default_rng(T + m)
