@@ -337,19 +337,25 @@ __device__ __forceinline__ void decode_prefetch(const DecodeArgs& a) {
 
 // GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
 // MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
-// STREAM: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
-// per pair it touches (slot warp + pair).  Else (split form) n_groups CTAs of their own work on each pair and leave a partial
-// state each.  A merge kernel joins the states, but for plain reads with one CTA per pair, which write the output.
-template <int D, int GP, bool MASS, bool STREAM>
-__global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_constant__ DecodeArgs a) {
+// FORM kStream: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
+// per pair it touches (slot warp + pair).  kSplit: n_groups CTAs of their own work on each pair and leave a partial state
+// each.  kSplitSmall: one CTA per pair with 4, 2 or 1 warps, several on an SM, where there are more pairs than SMs.  A merge kernel joins the states, but for plain reads with one CTA per pair, which write the output.
+enum DecodeForm { kStream, kSplit, kSplitSmall };
+constexpr int kDecSmallWarps = 4;  // of a kSplitSmall CTA at most
+// Warps an SM holds of kSplitSmall: 12 rings of 16 KB and 168 registers, 8 with the registers of 8 query heads at d = 128.
+constexpr int decode_small_warps_per_sm(int D, int GP) { return D == 128 && GP == 8 ? 8 : 12; }
+template <int D, int GP, bool MASS, DecodeForm FORM>
+__global__ void __launch_bounds__(FORM == kSplitSmall ? kDecSmallWarps * 32 : kDecThreads,
+                                  FORM == kSplitSmall ? decode_small_warps_per_sm(D, GP) / kDecSmallWarps : 1)
+decode_kernel(const __grid_constant__ DecodeArgs a) {
   using State = DecodeState<D, GP>;
-  constexpr int NT = kDecThreads, NW = kDecWarps;
+  const int NW = FORM == kSplitSmall ? (int)(blockDim.x >> 5) : kDecWarps, NT = NW * 32;
   constexpr int NCH = State::NCH;
   constexpr int kStageBytes = 2 * kDecBlock * D * 2;
   constexpr int kStages = kDecRingBytes / kStageBytes;
   extern __shared__ __align__(16) uint8_t dec_smem[];     // per-warp rings
 
-  if constexpr (!STREAM && !MASS)
+  if constexpr (FORM == kSplit && !MASS)
     if (a.prefetch) decode_prefetch<D>(a);
   pdl_wait();
   pdl_launch_dependents();
@@ -409,7 +415,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
   State st;
   st.clear();
 
-  if constexpr (STREAM) {
+  if constexpr (FORM == kStream) {
     const int nb = (n + kDecBlock - 1) / kDecBlock;       // blocks per pair
     const int total = a.pairs * nb;
     const int per = (total + a.n_warps - 1) / a.n_warps;
@@ -464,7 +470,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
       }
     }
   } else {
-    __shared__ float s_ml[NW][GP][2];
+    __shared__ float s_ml[FORM == kSplitSmall ? kDecSmallWarps : kDecWarps][GP][2];
     const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
     const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
     const int share = decode_share(n, a.n_groups);
@@ -500,7 +506,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_kernel(const __grid_con
     for (int t = threadIdx.x; t < G * V4; t += NT) {
       const int g = t / V4, e0 = (t - g * V4) * 4;
       float mm = -INFINITY, ll = 0.f, aa[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
+#pragma unroll (FORM == kSplitSmall ? 1 : kDecWarps)
       for (int w = 0; w < NW; ++w) {
         const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(dec_smem + w * kDecRingBytes) + g * D + e0);
         const float a2[4] = {v.x, v.y, v.z, v.w};
@@ -669,40 +675,54 @@ size_t decode_mass_ws_bytes(int n_layers, int Hkv, int Hq, int d, int n_cap) {
 // in a captured step (27.3 us with 512-key splits and 16-byte loads into registers; a cluster of 16 CTAs per pair with
 // the merge through distributed shared memory 24 us, since only 7 such clusters fit at a time; the last CTA of a pair
 // merging, found by an atomic count, 18.5 us).
+// More pairs than SMs, and too few keys to stream: CTAs of four, two or one warps, the most with which all of them run at
+// once.  Eight warps a CTA hold an SM to themselves: 64 layers x 32 heads x 64 rows, G = 1: 45.0 -> 21.1 us; 40 layers x 32
+// heads x 300 rows 51.3 -> 37.8; 40 layers x 8 heads x 300 rows, G = 4: 19.9 -> 15.6; 20 layers x 8 heads x 2500 rows 47.6
+// -> 42.8 (the CUDA-core kernel with 512-key splits: 21.6, 42.8, 23.7, 57.2).  Where not even one-warp CTAs run at once, four
+// warps are the best for longer pairs (2048 pairs x 512 rows: 86 us, two warps 90, one 103) and two for shorter (x 150:
+// 37.5, 35.2, 37.2).
 struct DecodePlan {
   int n_warps;       // > 0: stream form with that many warps
   int groups;        // else CTAs per pair
+  int small;         // > 0: one CTA per pair, of that many warps (kSplitSmall)
 };
-static DecodePlan decode_plan(int pairs, int n_cap, int n_sm) {
-  DecodePlan p{0, 1};
+static DecodePlan decode_plan(int pairs, int n_cap, int n_sm, int small_warps_per_sm) {
+  DecodePlan p{0, 1, 0};
   const int splits = std::max(1, (n_cap + kDecSplitKeys - 1) / kDecSplitKeys);  // partial slots per pair
   // stream form: warps + pairs slots
   const int warps = std::min(n_sm * kDecWarps, pairs * (splits - 1) / kDecWarps * kDecWarps);
   if (warps >= n_sm * kDecWarps * 3 / 4) p.n_warps = warps;
-  else p.groups = std::max(1, std::min(splits, n_sm / pairs));
+  else if (pairs <= n_sm) p.groups = std::min(splits, n_sm / pairs);
+  else if (pairs > n_sm * small_warps_per_sm) p.small = n_cap > 256 ? 4 : 2;
+  else
+    for (p.small = kDecSmallWarps; n_sm * (small_warps_per_sm / p.small) < pairs;) p.small /= 2;
   return p;
 }
 
-template <int D, int GP, bool MASS, bool STREAM>
-static cudaError_t decode_launch(const DecodeArgs& a, cudaStream_t stream) {
-  void (*kern)(DecodeArgs) = decode_kernel<D, GP, MASS, STREAM>;
-  const int smem = kDecWarps * kDecRingBytes;
-  const int grid = STREAM ? a.n_warps / kDecWarps : a.pairs * a.n_groups;
+template <int D, int GP, bool MASS, DecodeForm FORM>
+static cudaError_t decode_launch(const DecodeArgs& a, int warps, cudaStream_t stream) {
+  void (*kern)(DecodeArgs) = decode_kernel<D, GP, MASS, FORM>;
+  const int smem = warps * kDecRingBytes;
+  const int grid = FORM == kStream ? a.n_warps / kDecWarps : a.pairs * a.n_groups;
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), smem);
   // Both kernels launch dependently (each waits for the one before it before it uses anything that may still be
   // written): a captured decode step of 32 one-layer calls took 390 us when neither did anything before its wait, 406
   // with the first launched plainly, 541 with both; with the prefetch and the merge's dry run it takes 307.
-  if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(kDecThreads), smem, stream, a, true);
-  if (e != cudaSuccess || (!STREAM && !MASS && a.n_groups == 1)) return e;
+  if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(warps * 32), smem, stream, a, true);
+  if (e != cudaSuccess || (FORM != kStream && !MASS && a.n_groups == 1)) return e;
   const int blocks = a.pairs * (a.G + (MASS ? a.chunks : 0));
   return launch_kernel(decode_merge_kernel<D, MASS>, dim3(blocks), dim3(kDecMergeThreads), 0, stream, a, true);
 }
 
+template <int D, int GP, bool MASS>
+static cudaError_t decode_dispatch_form(const DecodeArgs& a, int small, cudaStream_t stream) {
+  if (a.n_warps > 0) return decode_launch<D, GP, MASS, kStream>(a, kDecWarps, stream);
+  return small > 0 ? decode_launch<D, GP, MASS, kSplitSmall>(a, small, stream)
+                   : decode_launch<D, GP, MASS, kSplit>(a, kDecWarps, stream);
+}
 template <int D, int GP>
-static cudaError_t decode_dispatch(const DecodeArgs& a, cudaStream_t stream) {
-  if (a.n_warps > 0)
-    return a.logits ? decode_launch<D, GP, true, true>(a, stream) : decode_launch<D, GP, false, true>(a, stream);
-  return a.logits ? decode_launch<D, GP, true, false>(a, stream) : decode_launch<D, GP, false, false>(a, stream);
+static cudaError_t decode_dispatch(const DecodeArgs& a, int small, cudaStream_t stream) {
+  return a.logits ? decode_dispatch_form<D, GP, true>(a, small, stream) : decode_dispatch_form<D, GP, false>(a, small, stream);
 }
 
 stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const* K, const void* const* V,
@@ -738,11 +758,11 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
     a.head_stride = head_stride;
     a.Hkv = Hkv;
     a.G = G;
-    const DecodePlan p = decode_plan(nl * Hkv, n_cap, n_sm);
+    const DecodePlan p = decode_plan(nl * Hkv, n_cap, n_sm, decode_small_warps_per_sm(d, G <= 4 ? 4 : 8));
     a.pairs = nl * Hkv;
     a.n_groups = p.groups;
     a.n_warps = p.n_warps;
-    a.prefetch = 2 * a.pairs * p.groups >= n_sm && (int64_t)(n_cap / p.groups) * (4 * d) > kDecWarps * kDecRingBytes;
+    a.prefetch = p.small == 0 && 2 * a.pairs * p.groups >= n_sm && (int64_t)(n_cap / p.groups) * (4 * d) > kDecWarps * kDecRingBytes;
     a.chunks = std::max(1, std::min(8, (n_cap + 1023) / 1024));
     a.n_dev = n_dev;
     a.n_host = n_host;
@@ -751,9 +771,9 @@ stepkv_status_t decode_run(int n_layers, const void* const* q, const void* const
     a.part = part;
     a.status = status;
     if (d == 128)
-      e = G <= 4 ? decode_dispatch<128, 4>(a, stream) : decode_dispatch<128, 8>(a, stream);
+      e = G <= 4 ? decode_dispatch<128, 4>(a, p.small, stream) : decode_dispatch<128, 8>(a, p.small, stream);
     else
-      e = G <= 4 ? decode_dispatch<64, 4>(a, stream) : decode_dispatch<64, 8>(a, stream);
+      e = G <= 4 ? decode_dispatch<64, 4>(a, p.small, stream) : decode_dispatch<64, 8>(a, p.small, stream);
     if (e != cudaSuccess) {
       set_last_cuda_error(e);
       return STEPKV_ECUDA;

@@ -132,6 +132,33 @@ def test_decode_stream_split(B, G, d, h2o, n):
         assert not mass[0][:, n:].any()
 
 
+@pytest.mark.parametrize("L,Hkv", [(5, 32), (16, 32), (40, 32), (64, 40)])
+@pytest.mark.parametrize("G,d,n", [(1, 128, 1), (1, 128, 130), (4, 128, 17), (5, 128, 300), (8, 64, 33), (2, 64, 500)])
+def test_decode_more_pairs_than_sms(B, L, Hkv, G, d, n):
+    """160 to 2560 (layer, KV head) pairs of few rows: one CTA of four, two or one warps per pair, several on an SM, with
+    warps that get no key, one block or a remainder.  Rows past n hold NaN."""
+    import torch
+    rng = np.random.default_rng(L + n + d)
+    rows = n + 7
+    some = [(_bits(rng, (Hkv * G, d), 2.0), _bits(rng, (Hkv, n, d)), _bits(rng, (Hkv, n, d))) for _ in range(3)]
+    pad = lambda x: torch.cat([TL.bf16_dev(x), torch.full((Hkv, rows - n, d), float("nan"), dtype=torch.bfloat16,
+                                                          device="cuda")], 1)
+    q, K, V = ([f(s[i]) for s in some] for i, f in enumerate((TL.bf16_dev, pad, pad)))
+    st = B.new_status()
+    args = [[x[l % 3] for l in range(L)] for x in (q, K, V)]
+    out = B.stepkv_decode(*args, n, status=st)
+    mass = [torch.zeros((Hkv, rows), dtype=torch.float32, device="cuda") for _ in range(L)]
+    same = B.stepkv_decode_h2o(*args, n, mass, status=st)
+    torch.cuda.synchronize()
+    assert st.item() == 0
+    for l in range(3):
+        TL.assert_decode_close(out[l].cpu().numpy(), *some[l], f"layer {l}")
+        TL.assert_close(mass[l][:, :n].cpu().numpy(), O.decode_attention_mass(some[l][0], some[l][1]), "mass", floor=1e-30)
+    for l in range(L):
+        assert torch.equal(out[l], out[l % 3]) and torch.equal(same[l], out[l]), l
+        assert torch.equal(mass[l], mass[l % 3]) and not mass[l][:, n:].any()
+
+
 @pytest.mark.parametrize("Hkv,d,rows", [(2, 128, 60), (2, 64, 600), (8, 128, 8911)])
 def test_decode_chain_with_changing_n(B, Hkv, d, rows):
     """Calls in a row whose number of keys is written on the device just before each: a call that starts fetching while
