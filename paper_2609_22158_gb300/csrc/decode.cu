@@ -19,17 +19,18 @@
 // at 8272 rows (5.2e-7 with fp32 FMAs and a logit rounded before its exponent).
 // Each warp copies whole rows (16 keys and values a step) into a ring of its own with cp.async and needs no other
 // warp: 13 instructions per key row instead of 79, so the reads bound it.  32 layers x 8 heads x 8272 rows, G = 4:
-// 208 -> 168 us (6.44 TB/s); 8 query heads per KV head 449 -> 172 us.  Reading the fragments straight from global
+// 208 -> 164 us (6.6 TB/s, the rate of a large copy); 8 query heads per KV head 449 -> 172 us.  Reading the fragments straight from global
 // memory, 64 bytes of each of 8 rows per load, ran at 215 us: full 128-byte lines matter.
 //
 // Two splits, chosen by the number of (layer, KV head) pairs and keys (decode_plan): each warp streams an equal range
 // of the list of all pairs' 16-key blocks, or (few pairs or keys) each pair is split over CTAs whose warps
-// interleave its blocks.  A second kernel merges the partial states of a pair in key order (deterministic).
+// interleave its blocks.  A second kernel merges the partial states of a pair in key order (deterministic); where one CTA
+// takes a whole pair there is none.
 // The number of keys may be read on the device (n_kept of a compaction), so no host sync is needed.
 //
 // Accumulated attention (the H2O-style token saliency, Sec. 4.2: T_i may come from an existing
 // token-level importance estimator): with mass rows given, the first kernel also stores every key's logits, and
-// the second adds (1/G) sum_g softmax_j(q_g . k_j / sqrt(d)) to mass[j] for each key from the heads' log-sum-exp:
+// the second (or the pair's one CTA) adds (1/G) sum_g softmax_j(q_g . k_j / sqrt(d)) to mass[j] for each key from the heads' log-sum-exp:
 // one writer per element and call, a fixed order over g, so the result is deterministic.
 #include <math.h>
 
@@ -335,11 +336,45 @@ __device__ __forceinline__ void decode_prefetch(const DecodeArgs& a) {
   if (r1 > r0) bulk_prefetch_l2(base + (size_t)(k_begin + r0) * D, (uint32_t)(r1 - r0) * 2 * D);
 }
 
+// Adds the group-mean softmax weight of keys [j0, j1) of a pair to its masses, from the stored logits and the heads'
+// log-sum-exp (one writer per key).  A chain of L2 loads, so four keys of a thread go at a time (25 layers x 32 heads x 1500
+// rows, G = 1: 115.8 -> 106.7 us).
+__device__ __forceinline__ void decode_add_mass(const DecodeArgs& a, int pair, const float* s_lse, int j0, int j1) {
+  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv, G = a.G;
+  const float inv_G = 1.f / (float)G;
+  float* mrow = a.mass[layer] + (size_t)h * a.mass_stride;
+  const float* lg = a.logits + (size_t)pair * a.n_cap * G;
+  constexpr int U = 4;  // keys of a thread in flight
+#pragma unroll 1
+  for (int j = j0 + (int)threadIdx.x; j < j1; j += U * (int)blockDim.x) {
+    float sum[U], was[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      sum[u] = 0.f;
+      was[u] = j + u * (int)blockDim.x < j1 ? mrow[j + u * (int)blockDim.x] : 0.f;
+    }
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = j + u * (int)blockDim.x < j1 ? __ldcg(lg + (size_t)(j + u * (int)blockDim.x) * G + g) : 0.f;
+#pragma unroll
+      for (int u = 0; u < U; ++u) sum[u] += ex2_approx(fmaf(x[u], a.c, -s_lse[g]));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (j + u * (int)blockDim.x < j1) mrow[j + u * (int)blockDim.x] = was[u] + sum[u] * inv_G;
+  }
+}
+__device__ __forceinline__ float decode_lse(float m, float l) { return l > 0.f ? m + __log2f(l) : INFINITY; }
+
 // GP: head rows per group of A's rows, 4 (G <= 4: three split terms in one MMA) or 8 (two MMAs).
 // MASS: the accumulated-attention variant (a separate instantiation, so the plain decode keeps its registers).
 // FORM kStream: each warp streams an equal contiguous range of the list of all pairs' 16-key blocks and leaves a partial state
 // per pair it touches (slot warp + pair).  kSplit: n_groups CTAs of their own work on each pair and leave a partial state
-// each.  kSplitSmall: one CTA per pair with 4, 2 or 1 warps, several on an SM, where there are more pairs than SMs.  A merge kernel joins the states, but for plain reads with one CTA per pair, which write the output.
+// each.  kSplitSmall: one CTA per pair with 4, 2 or 1 warps, several on an SM, where there are more pairs than SMs.  A merge
+// kernel joins the states and adds to the masses; one CTA per pair does both itself (64 layers x 8 heads x 64 rows with
+// masses, G = 4: 17.0 -> 14.1 us, 300 rows 30.9 -> 28.4).
 enum DecodeForm { kStream, kSplit, kSplitSmall };
 constexpr int kDecSmallWarps = 4;  // of a kSplitSmall CTA at most
 // Warps an SM holds of kSplitSmall: 12 rings of 16 KB and 168 registers, 8 with the registers of 8 query heads at d = 128.
@@ -470,7 +505,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
       }
     }
   } else {
-    __shared__ float s_ml[FORM == kSplitSmall ? kDecSmallWarps : kDecWarps][GP][2];
+    __shared__ float s_ml[FORM == kSplitSmall ? kDecSmallWarps : kDecWarps][GP][2], s_lse[GP];
     const int pair = blockIdx.x / a.n_groups, grp = blockIdx.x - pair * a.n_groups;
     const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
     const int share = decode_share(n, a.n_groups);
@@ -512,7 +547,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
         const float a2[4] = {v.x, v.y, v.z, v.w};
         merge_state<4>(mm, ll, aa, s_ml[w][g][0], s_ml[w][g][1], a2);
       }
-      if (!MASS && a.n_groups == 1) {
+      if (a.n_groups == 1) {
         float o[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[e] = decode_output<D>(decode_quotient(aa[e], ll), ll, Vh, n, e0 + e);
@@ -524,6 +559,13 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
           dst[1] = ll;
         }
         *reinterpret_cast<float4*>(dst + 4 + e0) = make_float4(aa[0], aa[1], aa[2], aa[3]);
+      }
+      if (MASS && e0 == 0) s_lse[g] = decode_lse(mm, ll);
+    }
+    if constexpr (MASS) {
+      if (a.n_groups == 1) {
+        __syncthreads();  // also: this CTA's logits are written
+        decode_add_mass(a, pair, s_lse, 0, n);
       }
     }
   }
@@ -628,7 +670,6 @@ __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __
   pdl_wait();
   pdl_launch_dependents();
   const int rest = item - a.pairs * G, pair = rest / a.chunks, chunk = rest - pair * a.chunks;
-  const int layer = pair / a.Hkv, h = pair - layer * a.Hkv;
   decode_slots(a, pair, first, count);
   for (int g = warp; g < G; g += NW) {
     float mm = -INFINITY, ll = 0.f, none[1] = {0.f};
@@ -641,20 +682,13 @@ __global__ void __launch_bounds__(kDecMergeThreads) decode_merge_kernel(const __
       const float m2 = __shfl_xor_sync(0xffffffffu, mm, o), l2 = __shfl_xor_sync(0xffffffffu, ll, o);
       merge_state<1>(mm, ll, none, m2, l2, none);
     }
-    if (lane == 0) s_lse[g] = ll > 0.f ? mm + __log2f(ll) : INFINITY;
+    if (lane == 0) s_lse[g] = decode_lse(mm, ll);
   }
   __syncthreads();
   const int n = max(0, min(decode_n(a), a.n_cap));
-  const float inv_G = 1.f / (float)G;
-  float* mrow = a.mass[layer] + (size_t)h * a.mass_stride;
-  const float* lg = a.logits + (size_t)pair * a.n_cap * G;
   const int per = (n + a.chunks - 1) / a.chunks;
-  const int j0 = chunk * per, j1 = min(n, j0 + per);
-  for (int j = j0 + threadIdx.x; j < j1; j += kDecMergeThreads) {
-    float sum = 0.f;
-    for (int g = 0; g < G; ++g) sum += ex2_approx(fmaf(__ldcg(lg + (size_t)j * G + g), a.c, -s_lse[g]));
-    mrow[j] += sum * inv_G;
-  }
+  const int j0 = chunk * per;
+  decode_add_mass(a, pair, s_lse, j0, min(n, j0 + per));
 }
 
 size_t decode_ws_bytes(int n_layers, int Hkv, int Hq, int d, int n_cap) {
@@ -709,7 +743,7 @@ static cudaError_t decode_launch(const DecodeArgs& a, int warps, cudaStream_t st
   // written): a captured decode step of 32 one-layer calls took 390 us when neither did anything before its wait, 406
   // with the first launched plainly, 541 with both; with the prefetch and the merge's dry run it takes 307.
   if (e == cudaSuccess) e = launch_kernel(kern, dim3(grid), dim3(warps * 32), smem, stream, a, true);
-  if (e != cudaSuccess || (FORM != kStream && !MASS && a.n_groups == 1)) return e;
+  if (e != cudaSuccess || (FORM != kStream && a.n_groups == 1)) return e;
   const int blocks = a.pairs * (a.G + (MASS ? a.chunks : 0));
   return launch_kernel(decode_merge_kernel<D, MASS>, dim3(blocks), dim3(kDecMergeThreads), 0, stream, a, true);
 }

@@ -73,7 +73,7 @@ def test_h2o_mass_matches_oracle(B, Hkv, G, d, n, rows, L, reads, ks):
                                               (32, 8, 2, 64, 3000, 6000)])
 def test_h2o_outputs_are_stepkv_decodes_bits(B, L, Hkv, G, d, n, rows):
     """One CTA per pair (few rows, or more than half as many pairs as SMs), split pairs, and streamed ranges: the output is
-    the same bit for bit with and without accumulated attention."""
+    the same bit for bit with and without accumulated attention, and a second read adds the same masses again."""
     import torch
     gen = torch.Generator(device="cuda").manual_seed(n + L)
     rnd = lambda *s: [torch.randn(s, generator=gen, device="cuda", dtype=torch.bfloat16) for _ in range(L)]
@@ -82,11 +82,14 @@ def test_h2o_outputs_are_stepkv_decodes_bits(B, L, Hkv, G, d, n, rows):
     st = B.new_status()
     plain = B.stepkv_decode(q, K, V, n, status=st)
     out = B.stepkv_decode_h2o(q, K, V, n, mass, status=st)
+    first = [m.clone() for m in mass]
+    B.stepkv_decode_h2o(q, K, V, n, mass, status=st)
     torch.cuda.synchronize()
     assert st.item() == 0
     for l in range(L):
         assert torch.equal(out[l], plain[l]), l
-        assert torch.allclose(mass[l].sum(1), torch.ones(Hkv, device="cuda"), rtol=1e-5)
+        assert torch.allclose(first[l].sum(1), torch.ones(Hkv, device="cuda"), rtol=1e-5)
+        assert torch.equal(mass[l], 2 * first[l]) and not mass[l][:, n:].any()
 
 
 @pytest.mark.parametrize("L", [64, 65, 80])
