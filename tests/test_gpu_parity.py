@@ -367,9 +367,8 @@ def test_select_budgets(B, budget):
 def test_select_exact_on_shared_fp32_priorities(B, levels):
     """alpha=1, beta=0, no normalisation, one saliency row: the kernel ranks exactly the fp32 values
     it is given, so its retained set must equal the oracle's ranking of the same values bit for bit,
-    ties (few distinct levels) included.  ~100-130 tokens per level (150 and 200 levels over 20000
-    tokens) put the threshold bin on both sides of the 128 candidates the value-bin path resolves
-    directly; 2 and 7 levels take the radix fallback."""
+    ties (few distinct levels) included: from half the tokens at one level down to 20, over every CTA of the
+    cluster."""
     import torch
     T = 20000
     tr = wl.custom(9, L=1, Hq=1, Hkv=1, d=64, T=T, W=8, n_steps=12, budget=wl.Budget.ratio(3, 10))

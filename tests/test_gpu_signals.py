@@ -83,6 +83,28 @@ def test_step_signals_reject_unsorted_cues(B):
     assert np.isnan(g[4:]).all() and np.isfinite(g[:4]).all()  # every target that compares with step 4
 
 
+@pytest.mark.parametrize("bad", [59, 37])
+def test_step_signals_reject_unsorted_cues_in_a_cluster(B, bad):
+    """One target and 59 earlier steps, spread over a cluster of CTAs: a bad list of the target, or of an earlier step,
+    sets the status, and only the values that depend on it stay unwritten."""
+    import torch
+    steps = wl.synthetic_cues(8, 60)
+    cues, cnt = C.pack_cues(steps)
+    good = torch.from_numpy(cues.view(np.int32)).cuda(), torch.from_numpy(cnt).cuda()
+    want = B.stepkv_step_signals(*good, obs_sim=torch.full((60,), -7.0, device="cuda"))[2]
+    cues[bad, 0, [0, 1]] = cues[bad, 0, [1, 0]]
+    st = B.new_status()
+    gain, red, obs_sim = B.stepkv_step_signals(torch.from_numpy(cues.view(np.int32)).cuda(), good[1],
+                                               obs_sim=torch.full((60,), -7.0, device="cuda"), status=st)
+    torch.cuda.synchronize()
+    assert st.item() == B.STEPKV_EDATA
+    assert torch.isnan(gain).all() and torch.isnan(red).all()
+    written = torch.arange(60, device="cuda") == 59
+    if bad != 59:
+        written = torch.arange(60, device="cuda") != bad
+    assert torch.equal(obs_sim[written], want[written]) and (obs_sim[~written] == -7.0).all()
+
+
 def test_signals_drive_the_fused_pass(B):
     """Cue-derived signals (gain, red, obs_sim from the kernel; valid from the workload) go straight into
     stepkv_compress; the oracle takes its own cue-derived signals."""
